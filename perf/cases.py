@@ -434,13 +434,16 @@ def run(state):
 # What a pass cannot do without
 # ---------------------------------------------------------------------------
 
-# Share of the samples whose opacity is not zero (the SDF falls along the ray):
-# only these need a colour.
-OPAQUE = 0.3
+# Share of the samples in the box whose opacity is not zero (the SDF falls
+# along the ray): only these need a colour.  Shares of the rays that cross the
+# box: a training batch of the object or of the body, a view.
+OPAQUE = 0.5
+CROSS = dict(object=0.46, sphere=0.46, body=0.63, view=0.26)
 
 
 def work(case):
     kind, n, N = case["kind"], case["rays"], case["samples"]
+    inside = n * N * CROSS["view" if kind in ("view", "proposed", "two_pass") else case["scene"]]
     nodes = case["rx"] * case["ry"] * case["rz"]
     if case["layout"] == "bricks":
         nodes = 4096 * _stored(case)
@@ -455,19 +458,19 @@ def work(case):
     ray = 24 + 24
     if kind == "step":
         return {"bytes": nodes * (per_node + 16) + coeffs * (pb + 4) + n * (ray + 12),
-                "flops": n * N * (2 * sdf + OPAQUE * 3 * colour)}
+                "flops": inside * (2 * sdf + OPAQUE * 3 * colour)}
     if kind == "view":
         return {"bytes": nodes * per_node + coeffs * pb + n * ray,
-                "flops": n * N * (sdf + OPAQUE * colour)}
+                "flops": inside * (sdf + OPAQUE * colour)}
     if kind == "proposed":
         return {"bytes": nodes * per_node + coeffs * pb + n * ray,
-                "flops": n * (N * (sdf + OPAQUE * colour) + prop)}
+                "flops": inside * (sdf + OPAQUE * colour) + n * prop}
     if kind == "two_pass":
         near = min(1.0, 3 * case["band"])
         return {"bytes": nodes * (per_node + 8) + coeffs * pb + n * ray,
-                "flops": nodes * near * colour + n * N * (sdf + OPAQUE * 48)}
+                "flops": nodes * near * colour + inside * (sdf + OPAQUE * 48)}
     if kind == "proposal":
-        return {"bytes": nodes * 4 + n * (24 + 8 * B + 4), "flops": n * (N * sdf + 3 * prop)}
+        return {"bytes": nodes * 4 + n * (24 + 8 * B + 4), "flops": inside * sdf + n * 3 * prop}
     # raw SDF, moments and their updates; s written; d s in and out; d s_hat
     tex = (nodes * 9) if case["layout"] == "planes" else 0
     return {"bytes": nodes * (4 + 4 + 8 + 24) + 3 * tex + 12 * coeffs,
