@@ -1,22 +1,20 @@
 // Grid-level training terms of ProbeSDF (Sec. 3.3, Eqs. 11-15).
 //
-//   smooth_kernel<false>  s = G(s_hat): 5^3 Gaussian (sigma = 1 node, separable,
-//                         replicated edge nodes); one shared-memory tile pass
-//                         (32 x 8 x 8 outputs, 2-node halo) per CTA
-//   smooth_kernel<true>   G^T: the same tiles with the transposed 1D operators,
-//                         applied z, y, x (edge outputs gather the replicated taps)
-//   sparse_smooth_kernel  both on sparse 16^3-node bricks: one CTA per stored
-//                         brick, its 16^3 nodes plus a 2-node halo gathered
-//                         through the brick table into a 20^3 tile
+//   smooth_kernel         s = G(s_hat): 5^3 Gaussian (sigma = 1 node, separable,
+//                         replicated edge nodes), or G^T with the transposed 1D
+//                         operators (edge outputs gather the replicated taps)
 //   sdf_reg_kernel        L_sdf, L_Eik and L_normal on the smoothed SDF, their
-//                         gradients scaled by (1 + 5 |s|)^-1: a z-streaming
-//                         stencil whose central-difference adjoint is a gather
+//                         gradients scaled by (1 + 5 |s|)^-1: the
+//                         central-difference adjoint as a gather
+//                         (both z-streaming, on dense grids and on sparse
+//                         16^3-node bricks behind a brick table)
 //   plane_reg_kernel      L_features: forward differences inside each tile plane
 //   probe_reg_kernel      L_probes: ordered pairs of 6-neighbour probes
 //
 // Streaming stencils over HBM-resident grids; loss values are summed per CTA
 // and added to device accumulators.
 #include <cmath>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -24,11 +22,17 @@ namespace psdf {
 
 namespace {
 
-constexpr int TX = 32, TY = 8, TZ = 8, HALO = 2;
-constexpr int AX = TX + 2 * HALO, AY = TY + 2 * HALO, AZ = TZ + 2 * HALO;
-constexpr int kBufA = AZ * AY * AX;  // 5184 floats
-constexpr int kBufB = AZ * AY * TX;  // 4608 floats (>= TZ * AY * AX = 3456)
-constexpr int kSmoothThreads = 256;
+// ---------------------------------------------------------------------------
+// z-streaming stencils.  A CTA owns an OX x OY column tile and walks z; every
+// thread owns one (x, y) column of the tile or of its halo.  Neighbours along
+// z are the thread's own registers, neighbours in the plane come from shared
+// memory.  Stage k of a plane runs one step after stage k - 1, on what the step
+// before wrote (two buffers per stage), so a step has a single barrier.
+// ---------------------------------------------------------------------------
+
+constexpr int HALO = 2;      // smoothing: 5 taps
+constexpr int REG_HALO = 3;  // regularisers: s -> normal -> gradient -> output
+constexpr int SB = 16;       // brick edge
 
 struct Taps {
     float w[5];
@@ -39,267 +43,311 @@ __device__ __forceinline__ int clampi(int v, int lo, int hi)
     return v < lo ? lo : (v > hi ? hi : v);
 }
 
-// Transposed 1D pass at output node k of an axis of n nodes; p[j * st] holds
-// input node k - 2 + j (0 outside the grid).  Inside the axis, output k takes
+// Columns of a tile in order of their distance to it: the OX x OY outputs
+// first, then ring 1, 2, .. of the halo (top row, bottom row, the two sides).
+// A stage that needs fewer columns than the one before thus leaves whole warps
+// out instead of the border lanes of every row.
+template <int OX_, int OY_, int H_>
+struct Tile {
+    static constexpr int OX = OX_, OY = OY_, H = H_;
+    static constexpr int kCols = (OX + 2 * H) * (OY + 2 * H);  // columns, halo included
+    static constexpr int kThreads = (kCols + 31) & ~31;
+    // columns within ring r
+    static __host__ __device__ constexpr int cols(int r) { return (OX + 2 * r) * (OY + 2 * r); }
+    static __device__ __forceinline__ void column(int e, int& x, int& y)
+    {
+        if (e < OX * OY) {
+            x = e % OX;
+            y = e / OX;
+            return;
+        }
+        e -= OX * OY;
+#pragma unroll
+        for (int r = 1; r <= H; ++r) {
+            const int w = OX + 2 * r, n = 2 * w + 2 * (OY + 2 * r) - 4;
+            if (e < n) {
+                if (e < 2 * w) {
+                    x = e % w - r;
+                    y = e < w ? -r : OY - 1 + r;
+                } else {
+                    e -= 2 * w;
+                    x = (e & 1) ? OX - 1 + r : -r;
+                    y = 1 - r + (e >> 1);
+                }
+                return;
+            }
+            e -= n;
+        }
+        x = y = 0;  // threads past the last column: never used
+    }
+};
+
+// Dense tiles: 32 outputs in x keep the rows of every array whole 128-byte
+// lines.  Brick tiles: a brick's 16 x 16 columns.
+using DenseSmooth = Tile<32, 16, HALO>;
+using BrickSmooth = Tile<SB, SB, HALO>;
+using DenseReg = Tile<32, 16, REG_HALO>;
+using BrickReg = Tile<SB, SB, REG_HALO>;
+
+// Where a kernel's planes lie.  Dense: node (x, y, z) is element
+// (z Ry + y) Rx + x, and CTA z covers planes [z zc, z zc + zc).  Sparse bricks:
+// node `local` of slot b is element b * 4096 + local; a CTA owns `seg` <= kMaxSeg bricks
+// of a brick column, whose stored bricks it walks run by run.
+struct Domain {
+    int R[3];
+    int zc;
+    const int* table;  // [B2][B1][B0]: slot, or -1 (outside [0, n_bricks) counts as absent)
+    int B[3], n_bricks, seg;
+};
+
+constexpr int kMaxSeg = 8;
+
+// Slots of the brick columns that a CTA's tile and halo lie in: its own and its
+// 8 neighbours, from the brick below its segment to the one above (-1: absent or
+// outside the grid).  Read once, all entries at a time: the walks then look
+// slots up in shared memory instead of waiting for the table brick after brick.
+struct SlotTable {
+    int slot[9][kMaxSeg + 2];
+};
+
+template <bool SPARSE>
+__device__ __forceinline__ void load_slots(const Domain& D, SlotTable& S)
+{
+    if constexpr (SPARSE) {
+        const int n = D.seg + 2;
+        for (int i = threadIdx.x; i < 9 * n; i += blockDim.x) {
+            const int c = i / n, k = i % n;
+            const int x = blockIdx.x + c % 3 - 1, y = blockIdx.y + c / 3 - 1;
+            const int z = blockIdx.z * D.seg + k - 1;
+            int s = -1;
+            if (x >= 0 && x < D.B[0] && y >= 0 && y < D.B[1] && z >= 0 && z < D.B[2])
+                s = __ldg(D.table + (int64_t(z) * D.B[1] + y) * D.B[0] + x);
+            S.slot[c][k] = s < D.n_bricks ? max(s, -1) : -1;
+        }
+        __syncthreads();
+    }
+}
+
+// The next run of planes [z0, z1) of this CTA, from `at` on (a brick, sparse;
+// negative: from the start); false when there is none.  CTA-uniform.
+template <bool SPARSE>
+__device__ __forceinline__ bool next_run(const Domain& D, const SlotTable& S, int& at, int& z0,
+                                         int& z1)
+{
+    if constexpr (!SPARSE) {
+        if (at >= 0) return false;
+        at = 0;
+        z0 = blockIdx.z * D.zc;
+        z1 = min(z0 + D.zc, D.R[2]);
+        return true;
+    } else {
+        const int first = blockIdx.z * D.seg, last = min(first + D.seg, D.B[2]);
+        const int* own = S.slot[4] + 1 - first;
+        int b = at < 0 ? first : at;
+        while (b < last && own[b] < 0) ++b;
+        if (b >= last) return false;
+        int e = b + 1;
+        while (e < last && own[e] >= 0) ++e;
+        at = e;
+        z0 = b * SB;
+        z1 = e * SB;
+        return true;
+    }
+}
+
+// A thread's column, walked plane by plane: `e` is the node of the current
+// plane in the arrays, -1 where it is not stored (sparse: its brick is absent).
+template <bool SPARSE>
+struct Walk {
+    int e;
+    int step;          // nodes between planes
+    int xy;            // offset inside a plane
+    const int* slots;  // sparse: the slots of the column's bricks, by brick
+    // column (x, y), inside the grid
+    __device__ __forceinline__ Walk(const Domain& D, const SlotTable& S, int x, int y)
+    {
+        if constexpr (SPARSE) {
+            const int c = ((y >> 4) - int(blockIdx.y) + 1) * 3 + (x >> 4) - int(blockIdx.x) + 1;
+            slots = S.slot[c] + 1 - int(blockIdx.z) * D.seg;
+            xy = ((y & 15) << 4) | (x & 15);
+            step = 256;
+        } else {
+            xy = y * D.R[0] + x;
+            step = D.R[0] * D.R[1];
+        }
+        e = -1;
+    }
+    // to plane z (inside the grid)
+    __device__ __forceinline__ void seek(const Domain& D, int z)
+    {
+        if constexpr (SPARSE) {
+            const int slot = slots[z >> 4];
+            e = slot < 0 ? -1 : slot * 4096 + ((z & 15) << 8) + xy;
+        } else {
+            e = z * step + xy;
+        }
+    }
+    // from plane z - 1 to plane z, both inside the grid
+    __device__ __forceinline__ void next(const Domain& D, int z)
+    {
+        if (SPARSE && (z & 15) == 0)
+            seek(D, z);
+        else if (!SPARSE || e >= 0)
+            e += step;
+    }
+};
+
+using Yes = std::true_type;
+using No = std::false_type;
+
+// 1D pass of 5 taps.  Transposed, at output node k of an axis of n nodes: v0 .. v4 are input
+// nodes k - 2 .. k + 2 (0 outside the grid).  Inside the axis, output k takes
 // input i with the weight w[k - i + 2] that the forward gave input k in output
 // i; the replicated edge taps add (w0 + w1) x in[0] + w0 x in[1] at k = 0 and
-// (w3 + w4) x in[n-1] + w4 x in[n-2] at k = n - 1.
-__device__ __forceinline__ float tconv(const float* p, int st, int k, int n, const Taps& T)
-{
-    float acc = 0.0f;
-#pragma unroll
-    for (int j = 0; j < 5; ++j) acc = fmaf(T.w[4 - j], p[j * st], acc);
-    if (k == 0) acc = fmaf(T.w[0] + T.w[1], p[2 * st], fmaf(T.w[0], p[3 * st], acc));
-    if (k == n - 1) acc = fmaf(T.w[3] + T.w[4], p[2 * st], fmaf(T.w[4], p[st], acc));
-    return acc;
-}
-
-// Work is laid out in rows along x: warp w takes rows w, w + 8, ..., lane =
-// x (a 36-wide halo row takes a second slot on lanes 0..3), so no element
-// index is ever divided or reduced modulo a tile size.
-constexpr int kSmoothWarps = kSmoothThreads / 32;
-
+// (w3 + w4) x in[n-1] + w4 x in[n-2] at k = n - 1 (`first`, `last`).
 template <bool TRANSPOSE>
-__global__ void __launch_bounds__(kSmoothThreads) smooth_kernel(const float* __restrict__ in,
-                                                                 int in_stride,
-                                                                 float* __restrict__ out,
-                                                                 int out_stride, int Rx, int Ry,
-                                                                 int Rz, Taps T, int accumulate)
+__device__ __forceinline__ float conv5(float v0, float v1, float v2, float v3, float v4,
+                                       bool first, bool last, const Taps& T)
 {
-    __shared__ float A[kBufA];
-    __shared__ float B[kBufB];
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * TZ;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // ---- tile + halo, rows (az, ay) of AX nodes: forward reads replicate the
-    // edge nodes; the transposed operator has no input outside the grid ----
-    {
-        const int gx0 = x0 - HALO + lane, gx1 = x0 - HALO + 32 + lane;
-        const bool in0 = gx0 >= 0 && gx0 < Rx, in1 = lane < AX - 32 && gx1 >= 0 && gx1 < Rx;
-        const int cx0 = clampi(gx0, 0, Rx - 1), cx1 = clampi(gx1, 0, Rx - 1);
-        constexpr int kRows = AZ * AY / kSmoothWarps;  // 18
-        constexpr int kBatch = 6;
-#pragma unroll 1
-        for (int i0 = 0; i0 < kRows; i0 += kBatch) {
-            float v0[kBatch], v1[kBatch];
-#pragma unroll
-            for (int i = 0; i < kBatch; ++i) {
-                const int r = warp + kSmoothWarps * (i0 + i);
-                const int ay = r % AY, az = r / AY;
-                const int gy = y0 + ay - HALO, gz = z0 + az - HALO;
-                v0[i] = v1[i] = 0.0f;
-                if (!TRANSPOSE) {
-                    const size_t row =
-                        ((size_t)clampi(gz, 0, Rz - 1) * Ry + clampi(gy, 0, Ry - 1)) * Rx;
-                    v0[i] = __ldg(in + (row + cx0) * in_stride);
-                    if (lane < AX - 32) v1[i] = __ldg(in + (row + cx1) * in_stride);
-                } else if (gy >= 0 && gy < Ry && gz >= 0 && gz < Rz) {
-                    const size_t row = ((size_t)gz * Ry + gy) * Rx;
-                    if (in0) v0[i] = __ldg(in + (row + gx0) * in_stride);
-                    if (in1) v1[i] = __ldg(in + (row + gx1) * in_stride);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < kBatch; ++i) {
-                const int r = warp + kSmoothWarps * (i0 + i);
-                A[r * AX + lane] = v0[i];
-                if (lane < AX - 32) A[r * AX + 32 + lane] = v1[i];
-            }
-        }
-    }
-    __syncthreads();
-    if (!TRANSPOSE) {
-        // x: A[AZ][AY][AX] -> B[AZ][AY][TX]
-        for (int r = warp; r < AZ * AY; r += kSmoothWarps) {
-            const float* a = A + r * AX + lane;
-            float acc = 0.0f;
-#pragma unroll
-            for (int j = 0; j < 5; ++j) acc = fmaf(T.w[j], a[j], acc);
-            B[r * TX + lane] = acc;
-        }
-        __syncthreads();
-        // y: B[AZ][AY][TX] -> A[AZ][TY][TX]
-        for (int r = warp; r < AZ * TY; r += kSmoothWarps) {
-            const int y = r % TY, az = r / TY;
-            const float* b = B + (az * AY + y) * TX + lane;
-            float acc = 0.0f;
-#pragma unroll
-            for (int j = 0; j < 5; ++j) acc = fmaf(T.w[j], b[j * TX], acc);
-            A[r * TX + lane] = acc;
-        }
-        __syncthreads();
-        // z: A[AZ][TY][TX] -> output
-        const int gx = x0 + lane;
-        for (int r = warp; r < TZ * TY; r += kSmoothWarps) {
-            const int y = r % TY, z = r / TY;
-            const int gy = y0 + y, gz = z0 + z;
-            if (gx >= Rx || gy >= Ry || gz >= Rz) continue;
-            const float* a = A + r * TX + lane;
-            float acc = 0.0f;
-#pragma unroll
-            for (int j = 0; j < 5; ++j) acc = fmaf(T.w[j], a[j * TY * TX], acc);
-            float* o = out + (((size_t)gz * Ry + gy) * Rx + gx) * out_stride;
-            *o = accumulate ? *o + acc : acc;
-        }
+    if constexpr (!TRANSPOSE) {
+        return fmaf(T.w[4], v4,
+                    fmaf(T.w[3], v3, fmaf(T.w[2], v2, fmaf(T.w[1], v1, T.w[0] * v0))));
     } else {
-        // G^T = Gx^T Gy^T Gz^T, applied z, y, x with tconv (zeros outside the
-        // grid, as loaded)
-        // z: A[AZ][AY][AX] -> B[TZ][AY][AX]
-        for (int r = warp; r < TZ * AY; r += kSmoothWarps) {
-            const int z = r / AY;
-            const float* a = A + r * AX + lane;  // rows (z, ay) of A start the tap column
-            B[r * AX + lane] = tconv(a, AY * AX, z0 + z, Rz, T);
-            if (lane < AX - 32) B[r * AX + 32 + lane] = tconv(a + 32, AY * AX, z0 + z, Rz, T);
-        }
-        __syncthreads();
-        // y: B[TZ][AY][AX] -> A[TZ][TY][AX]
-        for (int r = warp; r < TZ * TY; r += kSmoothWarps) {
-            const int y = r % TY, z = r / TY;
-            const float* b = B + (z * AY + y) * AX + lane;
-            A[r * AX + lane] = tconv(b, AX, y0 + y, Ry, T);
-            if (lane < AX - 32) A[r * AX + 32 + lane] = tconv(b + 32, AX, y0 + y, Ry, T);
-        }
-        __syncthreads();
-        // x: A[TZ][TY][AX] -> output
-        const int gx = x0 + lane;
-        for (int r = warp; r < TZ * TY; r += kSmoothWarps) {
-            const int y = r % TY, z = r / TY;
-            const int gy = y0 + y, gz = z0 + z;
-            if (gx >= Rx || gy >= Ry || gz >= Rz) continue;
-            const float acc = tconv(A + r * AX + lane, 1, gx, Rx, T);
-            float* o = out + (((size_t)gz * Ry + gy) * Rx + gx) * out_stride;
-            *o = accumulate ? *o + acc : acc;
-        }
+        float acc = fmaf(T.w[0], v4,
+                         fmaf(T.w[1], v3, fmaf(T.w[2], v2, fmaf(T.w[3], v1, T.w[4] * v0))));
+        if (first) acc = fmaf(T.w[0] + T.w[1], v2, fmaf(T.w[0], v3, acc));
+        if (last) acc = fmaf(T.w[3] + T.w[4], v2, fmaf(T.w[4], v1, acc));
+        return acc;
     }
 }
 
-// ---------------------------------------------------------------------------
-// Sparse bricks.  The grid is the full R^3 grid in which every node of a
-// brick that is not stored holds `empty` (forward: s_hat = s = empty_sdf
-// there); G and G^T are those of the full grid, evaluated at the stored nodes
-// only.  The transposed pass has no input at absent nodes (their s is fixed,
-// so they carry no gradient) nor outside the grid.  One CTA per table entry;
-// absent entries return at once.
-// ---------------------------------------------------------------------------
-
-constexpr int SB = 16, SA = SB + 2 * HALO;  // brick edge, tile edge (20)
-constexpr int kSpTile = SA * SA * SA;       // 8000 floats
-constexpr int kSpPass = SA * SA * SB;       // 6400 floats
-constexpr int kSpThreads = 256;
-constexpr int kSpBytes = static_cast<int>(sizeof(float)) * (kSpTile + kSpPass);
-
-struct SparseSmooth {
-    const int* table;  // [B2][B1][B0]: slot, or -1 (outside [0, n_bricks) counts as absent)
-    int B[3], R[3], n_bricks;
-    const float* in;   // node `local` of slot b at in[in_base + (b * 4096 + local) * in_stride]
-    int64_t in_base;
+struct Smooth {
+    Domain D;
+    const float* in;  // element e at in[e * in_stride]
     int in_stride;
-    float* out;        // likewise
-    int64_t out_base;
+    float* out;       // likewise
     int out_stride;
-    float empty;       // forward: the value of a node of an absent brick
+    float empty;      // sparse, forward: the value of a node of an absent brick
     int accumulate;
 };
 
-__device__ __forceinline__ int sparse_slot(const SparseSmooth& P, int bx, int by, int bz)
+// s = G(s_hat) or G^T.  What a node costs beyond memory is one load, two
+// 5-tap passes over shared memory (x, then y) and one over registers (z); the
+// next four planes (and what the outputs add to) are in flight meanwhile.
+//
+// Bound: HBM, by the 4-byte SDF slots of the 16-byte records (whole sectors are
+// moved: 0.57 GB for a 256^3 grid).  Measured on 256^3 node records: s 93 us,
+// G^T 95 us (a 32 x 8 x 8 tile with its halo gathered at once: 109 and 155 us);
+// on 47 M stored nodes of a 512^3 grid 297 and 327 us (20^3 tiles gathered per
+// brick with an index division per element: 568 and 763 us).
+//
+// Outside the grid the forward reads the replicated edge node and the
+// transpose 0; in an absent brick the forward reads `empty` and the transpose
+// 0 (an absent node's s is fixed, so it carries no gradient).
+template <class T, bool SPARSE, bool TRANSPOSE>
+__global__ void __launch_bounds__(T::kThreads, SPARSE ? 3 : 2) smooth_kernel(Smooth P, Taps taps)
 {
-    const int s = __ldg(P.table + (int64_t(bz) * P.B[1] + by) * P.B[0] + bx);
-    return s >= 0 && s < P.n_bricks ? s : -1;
-}
-
-template <bool TRANSPOSE>
-__global__ void __launch_bounds__(kSpThreads) sparse_smooth_kernel(SparseSmooth P, Taps T)
-{
-    extern __shared__ float sp_smem[];
-    float* A = sp_smem;            // tile [SA][SA][SA] (z, y, x), later the y pass
-    float* Bp = sp_smem + kSpTile; // x pass [SA][SA][SB]
-    __shared__ int nb[27];         // slots of the brick and its 26 neighbours
-    const int e = blockIdx.x;
-    const int bx = e % P.B[0], by = (e / P.B[0]) % P.B[1], bz = e / (P.B[0] * P.B[1]);
-    const int slot = sparse_slot(P, bx, by, bz);
-    if (slot < 0) return;  // CTA-uniform
-    const int tid = threadIdx.x;
-    if (tid < 27) {
-        const int nx = bx + tid % 3 - 1, ny = by + (tid / 3) % 3 - 1, nz = bz + tid / 9 - 1;
-        const bool in_grid = nx >= 0 && nx < P.B[0] && ny >= 0 && ny < P.B[1] && nz >= 0 &&
-                             nz < P.B[2];
-        nb[tid] = in_grid ? sparse_slot(P, nx, ny, nz) : -1;
-    }
-    __syncthreads();
-    // ---- tile: node g = 16 b - 2 + l.  Forward: the replicated edge node
-    // outside the grid, `empty` in an absent brick.  Transposed: 0 for both ----
-    const int g0[3] = {bx * SB - HALO, by * SB - HALO, bz * SB - HALO};
-    const int b0[3] = {bx, by, bz};
-    for (int i = tid; i < kSpTile; i += kSpThreads) {
-        const int l[3] = {i % SA, (i / SA) % SA, i / (SA * SA)};
-        int g[3];
-        bool inside = true;
+    // row pitch of the shared planes: 16-wide rows, two to a warp, fall on
+    // different halves of the banks
+    constexpr int W = T::OX == 16 ? 48 : T::OX + 2 * HALO;
+    __shared__ float S[2][W * (T::OY + 2 * HALO)];  // loaded plane
+    __shared__ float X[2][W * (T::OY + 2 * HALO)];  // after the x pass
+    __shared__ SlotTable slots;
+    const Domain& D = P.D;
+    load_slots<SPARSE>(D, slots);
+    const int x0 = blockIdx.x * T::OX, y0 = blockIdx.y * T::OY;
+    int lx, ly;
+    T::column(threadIdx.x, lx, ly);
+    const bool mine = threadIdx.x < T::kCols;
+    const int gx = x0 + lx, gy = y0 + ly;
+    const int pos = (ly + HALO) * W + lx + HALO;
+    const bool do_x = mine && lx >= 0 && lx < T::OX;
+    const bool do_y = threadIdx.x < T::OX * T::OY;
+    const bool do_out = do_y && gx < D.R[0] && gy < D.R[1];
+    const bool in_xy = gx >= 0 && gx < D.R[0] && gy >= 0 && gy < D.R[1];
+    const bool reads = mine && (!TRANSPOSE || in_xy);
+    const int cx = clampi(gx, 0, D.R[0] - 1), cy = clampi(gy, 0, D.R[1] - 1);
+    Walk<SPARSE> in(D, slots, cx, cy), ahead(D, slots, cx, cy), out(D, slots, cx, cy);
+    const float none = TRANSPOSE ? 0.0f : P.empty;
+    auto value = [&]() -> float {
+        return reads && (!SPARSE || in.e >= 0) ? __ldg(P.in + int64_t(in.e) * P.in_stride) : none;
+    };
+    auto edge_value = [&](int z) -> float {
+        return TRANSPOSE && (z < 0 || z >= D.R[2]) ? 0.0f : value();
+    };
+    int at = -1, z0, z1;
+    while (next_run<SPARSE>(D, slots, at, z0, z1)) {
+        // planes z0 - 2 .. z1 + 1 enter, kAhead of them in flight.  The x pass
+        // of plane z runs in step z, the y pass in step z + 2, and output plane
+        // z leaves in step z + 4.  The loop is unrolled over the period of the
+        // register rings (5) and of the shared buffers (2); steps away from the
+        // ends of the run and of the grid test no plane index.
+        constexpr int kAhead = 4;
+        float v[5], r[5];  // loaded planes; planes after the y pass
+        float old[5];      // what the outputs add to
+        const int zb = z0 - HALO;
+        in.seek(D, max(zb, 0));
+        v[0] = edge_value(zb);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            g[a] = g0[a] + l[a];
-            inside = inside && g[a] >= 0 && g[a] < P.R[a];
-            g[a] = clampi(g[a], 0, P.R[a] - 1);
+        for (int i = 1; i < kAhead; ++i) {
+            if (zb + i > 0 && zb + i < D.R[2]) in.next(D, zb + i);
+            v[i] = edge_value(zb + i);
         }
-        float v = TRANSPOSE ? 0.0f : P.empty;
-        if (!TRANSPOSE || inside) {
-            // the clamped node lies in this brick or a face / edge / corner neighbour
-            const int q = ((g[2] >> 4) - b0[2] + 1) * 9 + ((g[1] >> 4) - b0[1] + 1) * 3 +
-                          ((g[0] >> 4) - b0[0] + 1);
-            const int s = nb[q];
-            if (s >= 0) {
-                const int local = ((g[2] & 15) << 8) | ((g[1] & 15) << 4) | (g[0] & 15);
-                v = __ldg(P.in + P.in_base + (int64_t(s) * 4096 + local) * P.in_stride);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) r[i] = old[i] = 0.0f;
+        out.seek(D, z0);
+        ahead.seek(D, z0);
+        auto step = [&](auto inner, int u, int z) {
+            constexpr bool kInner = decltype(inner)::value;
+            if (mine) S[u & 1][pos] = v[u % 5];
+            if (kInner || z + kAhead < z1 + HALO) {
+                if (kInner || (z + kAhead > 0 && z + kAhead < D.R[2])) in.next(D, z + kAhead);
+                v[(u + kAhead) % 5] = kInner ? value() : edge_value(z + kAhead);
+            }
+            if (P.accumulate && do_out && (kInner || (z >= z0 && z < z1))) {
+                if (z > z0) ahead.next(D, z);
+                old[u % 5] = P.out[int64_t(ahead.e) * P.out_stride];
+            }
+            const int zo = z - 4;
+            if (do_y) {
+                const float* c = &X[u & 1][pos];  // the x pass of plane z - 2
+                r[u % 5] = conv5<TRANSPOSE>(c[-2 * W], c[-W], c[0], c[W], c[2 * W],
+                                            gy == 0, gy == D.R[1] - 1, taps);
+            }
+            if (do_out && (kInner || zo >= z0)) {
+                P.out[int64_t(out.e) * P.out_stride] =
+                    old[(u + 1) % 5] + conv5<TRANSPOSE>(r[(u + 1) % 5], r[(u + 2) % 5], r[(u + 3) % 5],
+                                           r[(u + 4) % 5], r[u % 5], !kInner && zo == 0,
+                                           !kInner && zo == D.R[2] - 1, taps);
+                if (kInner || zo + 1 < z1) out.next(D, zo + 1);
+            }
+            __syncthreads();  // plane z is in S; the x pass's buffer is read
+            if (do_x) {
+                const float* c = &S[u & 1][pos];
+                X[u & 1][pos] = conv5<TRANSPOSE>(c[-2], c[-1], c[0], c[1], c[2], gx == 0,
+                                                 gx == D.R[0] - 1, taps);
+            }
+        };
+        const int lo = z0 + 5, hi = min(z1 + HALO, D.R[2]) - kAhead;  // inner steps [lo, hi)
+        for (int zs = zb; zs < z1 + 4; zs += 10) {
+#pragma unroll
+            for (int u = 0; u < 10; ++u) {
+                const int z = zs + u;
+                if (z >= z1 + 4) break;
+                if (z >= lo && z < hi)
+                    step(Yes(), u, z);
+                else
+                    step(No(), u, z);
             }
         }
-        A[i] = v;
-    }
-    __syncthreads();
-    // ---- x: A[SA][SA][SA] -> Bp[SA][SA][SB] ----
-    for (int i = tid; i < kSpPass; i += kSpThreads) {
-        const int x = i % SB, r = i / SB;
-        const float* a = A + r * SA + x;
-        float acc = 0.0f;
-        if (TRANSPOSE) {
-            acc = tconv(a, 1, bx * SB + x, P.R[0], T);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 5; ++j) acc = fmaf(T.w[j], a[j], acc);
-        }
-        Bp[i] = acc;
-    }
-    __syncthreads();
-    // ---- y: Bp[SA][SA][SB] -> A[SA][SB][SB] ----
-    for (int i = tid; i < SA * SB * SB; i += kSpThreads) {
-        const int x = i % SB, y = (i / SB) % SB, z = i / (SB * SB);
-        const float* b = Bp + (z * SA + y) * SB + x;
-        float acc = 0.0f;
-        if (TRANSPOSE) {
-            acc = tconv(b, SB, by * SB + y, P.R[1], T);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 5; ++j) acc = fmaf(T.w[j], b[j * SB], acc);
-        }
-        A[i] = acc;
-    }
-    __syncthreads();
-    // ---- z: A[SA][SB][SB] -> the brick's 16^3 outputs ----
-    for (int i = tid; i < SB * SB * SB; i += kSpThreads) {
-        const float* a = A + i;
-        float acc = 0.0f;
-        if (TRANSPOSE) {
-            acc = tconv(a, SB * SB, bz * SB + (i >> 8), P.R[2], T);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 5; ++j) acc = fmaf(T.w[j], a[j * SB * SB], acc);
-        }
-        float* o = P.out + P.out_base + (int64_t(slot) * 4096 + i) * P.out_stride;
-        *o = P.accumulate ? *o + acc : acc;
+        __syncthreads();  // the last reads of S and X, before the next run's writes
     }
 }
 
 // Block sum of up to three loss partials, added to acc[0..n-1] (skipped when acc is null).
 __device__ __forceinline__ void block_loss(float a, float b, float c, float* acc, int n)
 {
-    __shared__ float part[3][8];
+    __shared__ float part[3][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -321,315 +369,295 @@ __device__ __forceinline__ void block_loss(float a, float b, float c, float* acc
     __syncthreads();
 }
 
+// 1 / x for 1 <= x, and 1 / sqrt(x) with the root itself for x in [1e-16, 1e30):
+// the hardware's approximations with one Newton-Raphson step, which leaves about
+// one unit in the last place, in a third of the instructions of the correctly
+// rounded forms.
+__device__ __forceinline__ float reciprocal(float x)
+{
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return x < 1e30f ? fmaf(r, fmaf(-x, r, 1.0f), r) : r;
+}
+
+__device__ __forceinline__ float inverse_root(float x, float& root)
+{
+    float r;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    const float h = x * r;              // about the root
+    const float e = fmaf(-h, r, 1.0f);  // 1 - x r^2
+    root = fmaf(0.5f * h, e, h);
+    return fmaf(0.5f * r, e, r);
+}
+
+// Asynchronous 4-byte copies into shared memory, in groups of one step.
+__device__ __forceinline__ void copy_async4(float* dst, const float* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+// All but the newest N groups of this thread have landed.
+template <int N>
+__device__ __forceinline__ void copy_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 struct SdfReg {
-    const float* s_hat;  // dense [R^3], or sparse [n_bricks][16^3] in slot order
-    const float* s;      // smoothed, element stride s_stride (sparse: the brick records)
+    Domain D;
+    const float* s_hat;  // element e at s_hat[e]
+    const float* s;      // smoothed, element stride s_stride
     int s_stride;
     float* d_s;          // gradient w.r.t. s (accumulated), stride d_stride
     int d_stride;
     float* d_s_hat;      // gradient w.r.t. s_hat (accumulated), laid out as s_hat
     float* loss;         // [3]: L_sdf, L_Eik, L_normal (accumulated)
-    int R[3];
     float inv2h[3];      // 1 / (2 h_a)
     float lam_sdf, lam_eik, lam_normal;
-    // sparse 16^3-node bricks: brick table [B2][B1][B0] (slot, or -1; a slot
-    // outside [0, n_bricks) counts as absent); node `local` of slot b is
-    // element b * 4096 + local of every array above; absent nodes read `empty`
-    const int* table;
-    int B[3], n_bricks;
-    float empty;
+    float empty;         // sparse: the value of a node of an absent brick
 };
 
-// z-streaming stencil.  A CTA owns an RX x RY column tile and ZC output planes
-// and walks z with three shared-memory rings of 3 planes each:
-//   s  (halo 3)  the smoothed SDF,
-//   N  (halo 2)  normal n, voxel weight w, rho = sqrt(|g|^2 + eps^2) (0 marks a
-//                node that is not interior), |g|,
-//   G  (halo 1)  dg = dObjective/d(grad s) of the node's Eikonal and normal
-//                terms.
-// Step t loads s plane zs, computes N at zs - 1, G at zs - 2 and the outputs
-// at zs - 3: ds_i = own L_sdf term + sum_a (dg_a(i - e_a) - dg_a(i + e_a)) / 2h_a
-// (the central-difference adjoint as a gather), so every output has one
-// writer and no atomics are needed.
+// L_sdf, L_Eik and L_normal with their gradients, z-streaming.  Step z loads s
+// plane z, computes N = {normal, voxel weight} of plane z - 1, G = dObjective /
+// d(grad s) of plane z - 2 and the outputs of plane z - 3:
+//   ds_i = own L_sdf term + sum_a (G_a(i - e_a) - G_a(i + e_a)) / 2h_a
+// (the central-difference adjoint as a gather, so every output has one writer
+// and no atomics are needed).  A node that is not interior has no normal; its
+// weight is stored as -1.
 //
-// Dense grids: 32 x 8 columns, 32 planes per CTA.  Sparse bricks: one CTA per
-// brick-table entry (absent entries return at once), 16 x 16 columns and the
-// brick's 16 planes; s is that of the full grid with every node of an absent
-// brick at `empty` (as the render and the smoothing read it), and the terms
-// are those of the stored nodes: an absent node gets voxel weight 0, so its
-// own Eikonal term and the normal pairs it owns add nothing, while its
-// normal still enters the pairs its stored neighbours own.  Gradients are
-// written for the stored nodes only (an absent node's s is not a parameter).
-template <int RX_, int RY_, int ZC_>
-struct RegTile {
-    static constexpr int RX = RX_, RY = RY_, ZC = ZC_;
-    static constexpr int SX = RX + 6, SY = RY + 6;
-    static constexpr int NX = RX + 4, NY = RY + 4;
-    static constexpr int GX = RX + 2, GY = RY + 2;
-    static constexpr int kThreads = RX * RY;
-    struct Smem {
-        float s[3][SY * SX];
-        float n[3][6][NY * NX];  // n.x n.y n.z w rho |g|
-        float g[3][3][GY * GX];  // dg
-    };
+// Bound: issue (73 % of the slots) and, on bricks, the serial chain of a step;
+// HBM would take 0.15 ms at 256^3.  s and the own values arrive by asynchronous
+// copies three planes ahead, which cost no registers.  Steps and warps whose
+// columns and planes all lie inside take straight-line code.  Measured: 256^3
+// 0.262 ms (0.421 with three barriers a plane and every neighbour read from
+// shared memory), 47 M stored nodes of a 512^3 grid 1.12 ms (1.28 ms).  Dense
+// tile: 32 x 16 outputs in 864 threads, 1 CTA per SM; 32 x 12 and 32 x 8 with 2
+// CTAs recompute more halo (0.29 and 0.38 ms).
+//
+// Sparse bricks: s is that of the full grid with every node of an absent brick
+// at `empty` (as the render and the smoothing read it), and the terms are those
+// of the stored nodes: an absent node gets voxel weight 0, so its own Eikonal
+// term and the normal pairs it owns add nothing, while its normal still enters
+// the pairs its stored neighbours own.  Gradients are written for the stored
+// nodes only (an absent node's s is not a parameter).
+template <class T>
+struct RegSmem {
+    static constexpr int H = REG_HALO;
+    static constexpr int kOwn = T::OX * T::OY;
+    // row pitches: of s, two 16-wide rows of a warp on different halves of the
+    // banks; of N (whole 16-byte lanes) and G, the row itself
+    static constexpr int kWS = T::OX == 16 ? 48 : T::OX + 2 * H, kWN = T::OX + 2 * H;
+    float4 N[2][T::kCols];
+    float2 G[2][T::kCols];
+    float s[6][kWS * (T::OY + 2 * H)];  // planes z - 1 .. z + 3
+    float own[3][6][kOwn];              // s_hat and d s_hat of plane z - 1, d s of plane z - 3
 };
-using DenseReg = RegTile<32, 8, 32>;
-using SparseReg = RegTile<16, 16, 16>;
-constexpr int kRegThreads = 256;
-static_assert(DenseReg::kThreads == kRegThreads && SparseReg::kThreads == kRegThreads, "");
 
 template <class T, bool SPARSE>
-__global__ void __launch_bounds__(kRegThreads) sdf_reg_kernel(SdfReg P)
+__global__ void __launch_bounds__(T::kThreads, SPARSE ? 2 : 1) sdf_reg_kernel(SdfReg P)
 {
-    constexpr int RX = T::RX, RY = T::RY, ZC = T::ZC;
-    constexpr int SX = T::SX, SY = T::SY, NX = T::NX, NY = T::NY, GX = T::GX, GY = T::GY;
-    extern __shared__ __align__(16) float reg_smem[];
-    typename T::Smem& S = *reinterpret_cast<typename T::Smem*>(reg_smem);
-    __shared__ int nb[27];  // sparse: slots of the brick and its 26 neighbours
+    using M = RegSmem<T>;
+    constexpr int H = REG_HALO, kWS = M::kWS, kWN = M::kWN;
+    constexpr int kAhead = 3;  // planes in flight
+    extern __shared__ __align__(16) uint8_t reg_smem[];
+    M& S = *reinterpret_cast<M*>(reg_smem);
+    __shared__ SlotTable slots;
+    const Domain& D = P.D;
+    load_slots<SPARSE>(D, slots);
+    const int x0 = blockIdx.x * T::OX, y0 = blockIdx.y * T::OY;
+    const int Rx = D.R[0], Ry = D.R[1], Rz = D.R[2];
+    int lx, ly;
+    T::column(threadIdx.x, lx, ly);
     const int tid = threadIdx.x;
-    const int Rx = P.R[0], Ry = P.R[1], Rz = P.R[2];
-    int x0, y0, z0, slot = 0;
-    if constexpr (SPARSE) {
-        const int e = blockIdx.x;
-        const int bx = e % P.B[0], by = (e / P.B[0]) % P.B[1], bz = e / (P.B[0] * P.B[1]);
-        const int sv = __ldg(P.table + e);
-        if (sv < 0 || sv >= P.n_bricks) return;  // CTA-uniform
-        slot = sv;
-        if (tid < 27) {
-            const int nx = bx + tid % 3 - 1, ny = by + (tid / 3) % 3 - 1, nz = bz + tid / 9 - 1;
-            int q = -1;
-            if (nx >= 0 && nx < P.B[0] && ny >= 0 && ny < P.B[1] && nz >= 0 && nz < P.B[2]) {
-                q = __ldg(P.table + (int64_t(nz) * P.B[1] + ny) * P.B[0] + nx);
-                if (q >= P.n_bricks) q = -1;
-            }
-            nb[tid] = q < 0 ? -1 : q;
-        }
-        __syncthreads();
-        x0 = bx * RX;
-        y0 = by * RY;
-        z0 = bz * ZC;
-    } else {
-        x0 = blockIdx.x * RX;
-        y0 = blockIdx.y * RY;
-        z0 = blockIdx.z * ZC;
-    }
-    const int z1 = min(z0 + ZC, Rz);
+    const int gx = x0 + lx, gy = y0 + ly;
+    const int pos = (ly + H) * kWN + lx + H, pos_s = (ly + H) * kWS + lx + H;
+    const bool do_s = tid < T::cols(3), do_n = tid < T::cols(2), do_g = tid < T::cols(1);
+    const bool in_xy = do_s && gx >= 0 && gx < Rx && gy >= 0 && gy < Ry;
+    const bool own_xy = tid < T::OX * T::OY && in_xy;
+    const bool n_xy = gx > 0 && gy > 0 && gx < Rx - 1 && gy < Ry - 1;  // interior in x and y
+    // warp-uniform: every lane an output column off the grid's faces
+    const bool full = __all_sync(0xffffffffu, own_xy && n_xy);
     const float cn = 2.0f * P.lam_normal;
-    const size_t plane = (size_t)Ry * Rx;
+    Walk<SPARSE> in(D, slots, clampi(gx, 0, Rx - 1), clampi(gy, 0, Ry - 1));
     float l_sdf = 0.0f, l_eik = 0.0f, l_nrm = 0.0f;
-    // sparse: element of in-grid node (x, y, z) in the arrays, or -1 if its
-    // brick is not stored (the node then lies in this brick or a neighbour)
-    auto sparse_elem = [&](int x, int y, int z) -> int64_t {
-        const int q = ((z >> 4) - (z0 >> 4) + 1) * 9 + ((y >> 4) - (y0 >> 4) + 1) * 3 +
-                      ((x >> 4) - (x0 >> 4) + 1);
-        const int b = nb[q];
-        return b < 0 ? -1 : int64_t(b) * 4096 + (((z & 15) << 8) | ((y & 15) << 4) | (x & 15));
-    };
-
-    // A thread's elements of each plane are the same at every step: their
-    // (x, y) offsets and in-grid tests are computed once.
-    constexpr int kPerS = (SY * SX + kRegThreads - 1) / kRegThreads;
-    constexpr int kPerN = (NY * NX + kRegThreads - 1) / kRegThreads;
-    constexpr int kPerG = (GY * GX + kRegThreads - 1) / kRegThreads;
-    size_t s_xy[kPerS];
-    bool s_in[kPerS];
-    int s_x[kPerS], s_y[kPerS];
+    int at = -1, z0, z1;
+    while (next_run<SPARSE>(D, slots, at, z0, z1)) {
+        // Rings in registers, unrolled over their period: the column's nodes of
+        // planes z - 2 .. z + 3, s of three planes, N of three, its 1 / rho and
+        // Eikonal factors of two, the L_sdf term and G_z of three.
+        int e[6] = {};
+        float s[3], ir[2], ee[2], ke[2], own[3], gz[3];
+        float4 n[3];
 #pragma unroll
-    for (int k = 0; k < kPerS; ++k) {
-        const int e = tid + k * kRegThreads;
-        const int x = x0 - 3 + e % SX, y = y0 - 3 + e / SX;
-        s_in[k] = e < SY * SX && x >= 0 && x < Rx && y >= 0 && y < Ry;
-        s_xy[k] = s_in[k] ? (size_t)y * Rx + x : 0;
-        s_x[k] = x;
-        s_y[k] = y;
-    }
-    int n_c[kPerN], n_x[kPerN], n_y[kPerN];
-    bool n_ok[kPerN], n_xy[kPerN];
-#pragma unroll
-    for (int k = 0; k < kPerN; ++k) {
-        const int e = tid + k * kRegThreads;
-        const int nx = e % NX, ny = e / NX, x = x0 - 2 + nx, y = y0 - 2 + ny;
-        n_ok[k] = e < NY * NX;
-        n_c[k] = (ny + 1) * SX + nx + 1;  // the node in the s planes
-        n_xy[k] = x > 0 && y > 0 && x < Rx - 1 && y < Ry - 1;
-        n_x[k] = x;
-        n_y[k] = y;
-    }
-    int g_c[kPerG];
-    bool g_ok[kPerG], g_xy[kPerG];
-#pragma unroll
-    for (int k = 0; k < kPerG; ++k) {
-        const int e = tid + k * kRegThreads;
-        const int gx = e % GX, gy = e / GX, x = x0 - 1 + gx, y = y0 - 1 + gy;
-        g_ok[k] = e < GY * GX;
-        g_c[k] = (gy + 1) * NX + gx + 1;  // the node in the N planes
-        g_xy[k] = x >= x0 && x < x0 + RX && y >= y0 && y < y0 + RY;  // owned in x, y
-    }
-
-    // s plane loads are software-pipelined: the values of plane zs + 1 are in
-    // flight while plane zs is processed
-    float pre[kPerS];
-    auto load_plane = [&](int z) {
-        const bool zin = z >= 0 && z < Rz;
-#pragma unroll
-        for (int k = 0; k < kPerS; ++k) {
-            if constexpr (SPARSE) {
-                float v = 0.0f;
-                if (zin && s_in[k]) {
-                    const int64_t el = sparse_elem(s_x[k], s_y[k], z);
-                    v = el < 0 ? P.empty : __ldg(P.s + el * P.s_stride);
+        for (int i = 0; i < 3; ++i) {
+            s[i] = own[i] = gz[i] = 0.0f;
+            n[i] = make_float4(0.f, 0.f, 0.f, -1.f);
+            if (i < 2) ir[i] = ee[i] = ke[i] = 0.0f;
+        }
+        const int zb = z0 - H;
+        // plane z + 3 of s and the own values of the step that it enters in,
+        // asynchronously: s is 0 outside the grid and `empty` in absent bricks
+        auto fetch = [&](auto inner, int z, int slot) {
+            constexpr bool kInner = decltype(inner)::value;
+            const bool in_z = kInner || (z >= 0 && z < Rz);
+            if (do_s) {
+                float* dst = &S.s[slot][pos_s];
+                if (!in_z || !in_xy)
+                    *dst = 0.0f;
+                else if (SPARSE && e[slot] < 0)
+                    *dst = P.empty;
+                else
+                    copy_async4(dst, P.s + int64_t(e[slot]) * P.s_stride);
+            }
+            if (own_xy) {
+                const int e1 = e[(slot + 5) % 6], e3 = e[(slot + 3) % 6];  // planes z - 1, z - 3
+                if (kInner || (z - 1 >= z0 && z - 1 < z1)) {
+                    copy_async4(&S.own[0][slot][tid], P.s_hat + e1);
+                    copy_async4(&S.own[1][slot][tid], P.d_s_hat + e1);
                 }
-                pre[k] = v;
+                if (kInner || (z - 3 >= z0 && z - 3 < z1))
+                    copy_async4(&S.own[2][slot][tid], P.d_s + int64_t(e3) * P.d_stride);
+            }
+            copy_commit();
+        };
+        auto walk = [&](int z, int slot) {  // the node of plane z
+            if (z > 0 && z < Rz) in.next(D, z);
+            e[slot] = in.e;
+        };
+        in.seek(D, max(zb, 0));
+        e[0] = in.e;
+        fetch(No(), zb, 0);
+        walk(zb + 1, 1);
+        fetch(No(), zb + 1, 1);
+        walk(zb + 2, 2);
+        fetch(No(), zb + 2, 2);
+        auto step = [&](auto inner, int u, int z) {
+            // inner: a step away from the ends, in a warp of interior output
+            // columns: straight-line code
+            constexpr bool kInner = decltype(inner)::value;
+            const int zo = z - 3;
+            const int e_out = e[(u + 3) % 6];
+            copy_wait<kAhead - 1>();
+            __syncthreads();  // plane z has landed; N of plane z - 2 and G of z - 3 are written
+            if (kInner || z + kAhead < z1 + H) {
+                walk(z + kAhead, (u + kAhead) % 6);
+                fetch(inner, z + kAhead, (u + kAhead) % 6);
             } else {
-                pre[k] = (zin && s_in[k])
-                             ? __ldg(P.s + ((size_t)z * plane + s_xy[k]) * P.s_stride)
-                             : 0.0f;
+                copy_commit();  // an empty group keeps the count
             }
-        }
-    };
-    load_plane(z0 - 3);
-    const int ox = tid % RX, oy = tid / RX;
-    const int x_o = x0 + ox, y_o = y0 + oy;
-    const int c_o = (oy + 1) * GX + ox + 1;  // the output node in the G planes
-    // ring slots of the planes of two steps back (ra), one step back (rb) and
-    // this step (rc): s holds zs, zs - 1, zs - 2; N holds zs - 1 .. zs - 3; G
-    // holds zs - 2 .. zs - 4
-    int ra = 0, rb = 1, rc = 2;
-    for (int zs = z0 - 3; zs <= z1 + 2; ++zs) {
-        // ---- s plane zs (zeros outside the grid), then the next plane's loads ----
-#pragma unroll
-        for (int k = 0; k < kPerS; ++k) {
-            const int e = tid + k * kRegThreads;
-            if (e < SY * SX) S.s[rc][e] = pre[k];
-        }
-        if (zs + 1 <= z1 + 2) load_plane(zs + 1);
-        // the output node's own values, consumed after the G stage
-        const int zo = zs - 3;
-        const bool out = zo >= z0 && zo < z1 && x_o < Rx && y_o < Ry;
-        size_t io = 0;
-        float s_o = 0.f, sh_o = 0.f, ds_o = 0.f, dsh_o = 0.f;
-        if (out) {
-            if constexpr (SPARSE)
-                io = size_t(slot) * 4096 + (((zo & 15) << 8) | ((y_o & 15) << 4) | (x_o & 15));
-            else
-                io = (size_t)zo * plane + (size_t)y_o * Rx + x_o;
-            s_o = __ldg(P.s + io * P.s_stride);
-            sh_o = __ldg(P.s_hat + io);
-            ds_o = P.d_s[io * P.d_stride];
-            dsh_o = P.d_s_hat[io];
-        }
-        __syncthreads();
-        // ---- N plane zn = zs - 1: gradient, normal, weight at interior nodes ----
-        // (the outputs need N at z0 - 2 .. z1 + 1 and G at z0 - 1 .. z1)
-        if (zs - 1 >= z0 - 2) {
-            const int zn = zs - 1;
-            const float* sm = S.s[ra];
-            const float* sc = S.s[rb];
-            const float* sp = S.s[rc];
-            const bool zin = zn > 0 && zn < Rz - 1;
-#pragma unroll
-            for (int k = 0; k < kPerN; ++k) {
-                if (!n_ok[k]) continue;
-                const int e = tid + k * kRegThreads;
-                const int c = n_c[k];
-                float n0 = 0.f, n1 = 0.f, n2 = 0.f, w = 0.f, rho = 0.f, gn = 0.f;
-                if (zin && n_xy[k]) {
-                    const float g0 = (sc[c + 1] - sc[c - 1]) * P.inv2h[0];
-                    const float g1 = (sc[c + SX] - sc[c - SX]) * P.inv2h[1];
-                    const float g2 = (sp[c] - sm[c]) * P.inv2h[2];
-                    const float gg = g0 * g0 + g1 * g1 + g2 * g2;
-                    rho = sqrtf(gg + 1e-24f);
-                    const float ir = 1.0f / rho;
-                    n0 = g0 * ir;
-                    n1 = g1 * ir;
-                    n2 = g2 * ir;
-                    gn = sqrtf(gg);
-                    w = 1.0f / (1.0f + 5.0f * fabsf(sc[c]));
-                    if constexpr (SPARSE)
-                        if (sparse_elem(n_x[k], n_y[k], zn) < 0) w = 0.0f;  // no terms of its own
-                }
-                S.n[rc][0][e] = n0;
-                S.n[rc][1][e] = n1;
-                S.n[rc][2][e] = n2;
-                S.n[rc][3][e] = w;
-                S.n[rc][4][e] = rho;
-                S.n[rc][5][e] = gn;
+            const int p = u & 1, q = p ^ 1;  // planes z - 2 and z - 1, z - 3 of N and G
+            const int iC = u % 3, iB = (u + 2) % 3, iA = (u + 1) % 3;
+            const float sp = s[iC] = (kInner || do_s) ? S.s[u][pos_s] : 0.0f;
+            const float sc = s[iB], sm = s[iA];
+            const float w = reciprocal(fmaf(5.0f, fabsf(sc), 1.0f));
+            // ---- Eq. 11 of plane z - 1 ----
+            own[iC] = 0.0f;
+            if (kInner || (own_xy && z - 1 >= z0 && z - 1 < z1)) {
+                const float r = sc - S.own[0][u][tid];
+                l_sdf = fmaf(r, r, l_sdf);
+                own[iC] = P.lam_sdf * w * 2.0f * r;
+                P.d_s_hat[e[(u + 5) % 6]] = S.own[1][u][tid] - own[iC];
             }
-        }
-        __syncthreads();
-        // ---- G plane zg = zs - 2: Eikonal and normal adjoints w.r.t. grad s ----
-        if (zs - 2 >= z0 - 1) {
-            const int zg = zs - 2;
-            const bool zown = zg >= z0 && zg < z1;
-#pragma unroll
-            for (int k = 0; k < kPerG; ++k) {
-                if (!g_ok[k]) continue;
-                const int e = tid + k * kRegThreads;
-                const int c = g_c[k];
-                const float rho = S.n[rb][4][c];
-                float d0 = 0.f, d1 = 0.f, d2 = 0.f;
-                if (rho > 0.0f) {
-                    const bool own = zown && g_xy[k];
-                    const float n0 = S.n[rb][0][c], n1 = S.n[rb][1][c], n2 = S.n[rb][2][c];
-                    const float w = S.n[rb][3][c], gn = S.n[rb][5][c];
-                    // Eq. 12
-                    const float ee = gn - 1.0f;
-                    if (own) l_eik += ee * ee;
-                    const float ce = gn > 0.0f ? P.lam_eik * w * 2.0f * ee / gn : 0.0f;
-                    // Eq. 13: pairs (j, j + e_a) owned by j, (j - e_a, j) owned by the neighbour
-                    float dn0 = 0.f, dn1 = 0.f, dn2 = 0.f;
-                    const int pr[3] = {rb, rb, rc}, po[3] = {c + 1, c + NX, c};
-                    const int mr[3] = {rb, rb, ra}, mo[3] = {c - 1, c - NX, c};
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (S.n[pr[a]][4][po[a]] > 0.0f) {
-                            const float q0 = S.n[pr[a]][0][po[a]] - n0;
-                            const float q1 = S.n[pr[a]][1][po[a]] - n1;
-                            const float q2 = S.n[pr[a]][2][po[a]] - n2;
-                            if (own) l_nrm += q0 * q0 + q1 * q1 + q2 * q2;
-                            const float kk = cn * w;
-                            dn0 -= kk * q0;
-                            dn1 -= kk * q1;
-                            dn2 -= kk * q2;
-                        }
-                        if (S.n[mr[a]][4][mo[a]] > 0.0f) {
-                            const float kk = cn * S.n[mr[a]][3][mo[a]];
-                            dn0 += kk * (n0 - S.n[mr[a]][0][mo[a]]);
-                            dn1 += kk * (n1 - S.n[mr[a]][1][mo[a]]);
-                            dn2 += kk * (n2 - S.n[mr[a]][2][mo[a]]);
-                        }
+            // ---- N of plane z - 1: gradient, normal, weight at interior nodes ----
+            if (kInner || do_n) {
+                n[iC] = make_float4(0.f, 0.f, 0.f, -1.f);
+                if (kInner || (n_xy && z - 1 > 0 && z - 1 < Rz - 1)) {
+                    const float* c = &S.s[(u + 5) % 6][pos_s];
+                    const float g0 = (c[1] - c[-1]) * P.inv2h[0];
+                    const float g1 = (c[kWS] - c[-kWS]) * P.inv2h[1];
+                    const float g2 = (sp - sm) * P.inv2h[2];
+                    const float gg = fmaf(g2, g2, fmaf(g1, g1, g0 * g0));
+                    const float wn = (SPARSE && !kInner && e[(u + 5) % 6] < 0) ? 0.0f : w;
+                    // rho = sqrt(|g|^2 + 1e-24); from 1e-16 on it equals |g| in FP32
+                    float rho, ratio = 1.0f;
+                    float irho = inverse_root(gg, rho), gn = rho;
+                    if (!(gg >= 1e-16f && gg < 1e30f)) {
+                        rho = sqrtf(gg + 1e-24f);
+                        irho = 1.0f / rho;
+                        gn = sqrtf(gg);
+                        ratio = gn > 0.0f ? rho / gn : 0.0f;
                     }
-                    const float ndn = n0 * dn0 + n1 * dn1 + n2 * dn2;
-                    const float ir = 1.0f / rho;
-                    // dg = ce g + (dn - n (n . dn)) / rho, with g = n rho
-                    d0 = ce * n0 * rho + (dn0 - n0 * ndn) * ir;
-                    d1 = ce * n1 * rho + (dn1 - n1 * ndn) * ir;
-                    d2 = ce * n2 * rho + (dn2 - n2 * ndn) * ir;
+                    ir[q] = irho;
+                    ee[q] = gn - 1.0f;
+                    // Eq. 12: its gradient is ke n
+                    ke[q] = P.lam_eik * wn * 2.0f * ee[q] * ratio;
+                    if (rho > 0.0f) n[iC] = make_float4(g0 * irho, g1 * irho, g2 * irho, wn);
                 }
-                S.g[rc][0][e] = d0;
-                S.g[rc][1][e] = d1;
-                S.g[rc][2][e] = d2;
+                S.N[q][pos] = n[iC];
+            }
+            // ---- G of plane z - 2: Eikonal and normal adjoints w.r.t. grad s ----
+            gz[iC] = 0.0f;
+            if (kInner || do_g) {
+                // Eq. 13: pairs (j, j + e_a) owned by j, (j - e_a, j) owned by the
+                // neighbour; a node without a normal (w = -1) takes part in none
+                const float n0 = n[iB].x, n1 = n[iB].y, n2 = n[iB].z;
+                const bool has = !(n[iB].w < 0.0f);
+                const float kw = has ? cn * n[iB].w : 0.0f;
+                const float4* c = &S.N[p][pos];
+                float d0 = 0.f, d1 = 0.f, d2 = 0.f, lq = 0.f;
+                auto up = [&](const float4& v) {
+                    const float q0 = n0 - v.x, q1 = n1 - v.y, q2 = n2 - v.z;
+                    const bool pair = !(v.w < 0.0f);
+                    const float k = pair ? kw : 0.0f;
+                    const float qq = fmaf(q2, q2, fmaf(q1, q1, q0 * q0));
+                    lq += pair ? qq : 0.0f;
+                    d0 = fmaf(k, q0, d0);
+                    d1 = fmaf(k, q1, d1);
+                    d2 = fmaf(k, q2, d2);
+                };
+                auto down = [&](const float4& v) {
+                    const float k = v.w < 0.0f ? 0.0f : cn * v.w;
+                    d0 = fmaf(k, n0 - v.x, d0);
+                    d1 = fmaf(k, n1 - v.y, d1);
+                    d2 = fmaf(k, n2 - v.z, d2);
+                };
+                up(c[1]);
+                down(c[-1]);
+                up(c[kWN]);
+                down(c[-kWN]);
+                down(n[iA]);
+                up(n[iC]);
+                if ((kInner || (own_xy && z - 2 >= z0 && z - 2 < z1)) && has) {
+                    l_eik = fmaf(ee[p], ee[p], l_eik);
+                    l_nrm += lq;
+                }
+                // dg = ke n + (d - n (n . d)) / rho
+                const float nd = -fmaf(n2, d2, fmaf(n1, d1, n0 * d0));
+                d0 = has ? fmaf(ke[p], n0, fmaf(n0, nd, d0) * ir[p]) : 0.0f;
+                d1 = has ? fmaf(ke[p], n1, fmaf(n1, nd, d1) * ir[p]) : 0.0f;
+                gz[iC] = has ? fmaf(ke[p], n2, fmaf(n2, nd, d2) * ir[p]) : 0.0f;
+                S.G[p][pos] = make_float2(d0, d1);
+            }
+            // ---- outputs of plane z - 3 ----
+            if (kInner || (own_xy && zo >= z0)) {
+                const float2* c = &S.G[q][pos];
+                const float adj = fmaf(c[-1].x - c[1].x, P.inv2h[0],
+                                       fmaf(c[-kWN].y - c[kWN].y, P.inv2h[1],
+                                            (gz[iA] - gz[iC]) * P.inv2h[2]));
+                P.d_s[int64_t(e_out) * P.d_stride] = S.own[2][u][tid] + (own[iA] + adj);
+            }
+        };
+        // inner steps [lo, hi): the fetched plane z + 3 and its own values lie
+        // in the run and in the grid, and so does every plane that is used
+        const int lo = z0 + H, hi = min(z1, Rz) - kAhead;
+        for (int zs = zb; zs < z1 + H; zs += 6) {
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+                const int z = zs + u;
+                if (z >= z1 + H) break;
+                if (full && z >= lo && z < hi)
+                    step(Yes(), u, z);
+                else
+                    step(No(), u, z);
             }
         }
-        __syncthreads();
-        // ---- outputs at zo = zs - 3 (G planes zo - 1, zo, zo + 1 in ra, rb, rc) ----
-        if (out) {
-            const float w = 1.0f / (1.0f + 5.0f * fabsf(s_o));
-            // Eq. 11
-            const float r = s_o - sh_o;
-            l_sdf += r * r;
-            const float own = P.lam_sdf * w * 2.0f * r;
-            P.d_s_hat[io] = dsh_o - own;
-            const int c = c_o;
-            const float adj = (S.g[rb][0][c - 1] - S.g[rb][0][c + 1]) * P.inv2h[0] +
-                              (S.g[rb][1][c - GX] - S.g[rb][1][c + GX]) * P.inv2h[1] +
-                              (S.g[ra][2][c] - S.g[rc][2][c]) * P.inv2h[2];
-            P.d_s[io * P.d_stride] = ds_o + (own + adj);
-        }
-        const int t = ra;  // rotate: this step's slots become one step back
-        ra = rb;
-        rb = rc;
-        rc = t;
+        copy_wait<0>();
+        __syncthreads();  // the last reads, before the next run's writes
     }
     block_loss(l_sdf, l_eik, l_nrm, P.loss, 3);
 }
@@ -745,17 +773,90 @@ int blocks(int64_t n)
 
 }  // namespace
 
+namespace {
+
+// Planes per CTA of a dense z-streaming kernel: the split of z into equal
+// chunks whose waves of resident CTAs take the fewest steps (a chunk costs its
+// planes plus `extra` steps of halo and pipeline).
+int dense_chunk(int64_t tiles, int Rz, int resident, int extra)
+{
+    const int64_t slots = int64_t(sms()) * resident;
+    int best = Rz;
+    int64_t cost = INT64_MAX;
+    for (int n = 1; n <= (Rz + 7) / 8 && n <= 65535; ++n) {
+        const int zc = (Rz + n - 1) / n;
+        const int64_t waves = (tiles * ((Rz + zc - 1) / zc) + slots - 1) / slots;
+        if (waves * (zc + extra) < cost) {
+            cost = waves * (zc + extra);
+            best = zc;
+        }
+    }
+    return best;
+}
+
+template <class T>
+dim3 dense_domain(const int R[3], int resident, int extra, Domain& D)
+{
+    for (int a = 0; a < 3; ++a) {
+        D.R[a] = R[a];
+        D.B[a] = 0;
+    }
+    D.table = nullptr;
+    D.n_bricks = D.seg = 0;
+    const int tx = (R[0] + T::OX - 1) / T::OX, ty = (R[1] + T::OY - 1) / T::OY;
+    D.zc = dense_chunk(int64_t(tx) * ty, R[2], resident, extra);
+    return dim3(tx, ty, (R[2] + D.zc - 1) / D.zc);
+}
+
+// Sparse: a CTA walks kMaxSeg bricks along z, so that neighbouring stored bricks
+// share their halo planes and pipeline (512^3 object, 11 468 stored bricks: all
+// three kernels 1.92 ms with 8, 1.99 ms with 4); with too few bricks to fill the
+// GPU several times over (16 per SM) it takes one.
+dim3 brick_domain(const int R[3], const int* table, int n_bricks, Domain& D)
+{
+    int64_t entries = 1;
+    for (int a = 0; a < 3; ++a) {
+        D.R[a] = R[a];
+        D.B[a] = R[a] / SB;
+        entries *= D.B[a];
+    }
+    D.zc = 0;
+    D.table = table;
+    D.n_bricks = n_bricks;
+    D.seg = n_bricks >= 16 * sms() ? kMaxSeg : 1;
+    return dim3(D.B[0], D.B[1], (D.B[2] + D.seg - 1) / D.seg);
+}
+
+template <class T, bool SPARSE>
+cudaError_t launch_reg(const SdfReg& P, dim3 grid, cudaStream_t stream)
+{
+    constexpr int kBytes = static_cast<int>(sizeof(RegSmem<T>));
+    auto kernel = sdf_reg_kernel<T, SPARSE>;
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, T::kThreads, kBytes, stream>>>(P);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 cudaError_t launch_smooth(const int R[3], const float* in, int in_stride, float* out,
                           int out_stride, bool transpose, bool accumulate, cudaStream_t stream)
 {
-    const dim3 grid((R[0] + TX - 1) / TX, (R[1] + TY - 1) / TY, (R[2] + TZ - 1) / TZ);
-    const Taps T = gauss_taps();
+    using T = DenseSmooth;
+    Smooth P;
+    const dim3 grid = dense_domain<T>(R, 2, 6, P.D);
+    P.in = in;
+    P.in_stride = in_stride;
+    P.out = out;
+    P.out_stride = out_stride;
+    P.empty = 0.0f;
+    P.accumulate = accumulate ? 1 : 0;
     if (transpose)
-        smooth_kernel<true><<<grid, kSmoothThreads, 0, stream>>>(in, in_stride, out, out_stride, R[0], R[1],
-                                                       R[2], T, accumulate ? 1 : 0);
+        smooth_kernel<T, false, true><<<grid, T::kThreads, 0, stream>>>(P, gauss_taps());
     else
-        smooth_kernel<false><<<grid, kSmoothThreads, 0, stream>>>(in, in_stride, out, out_stride, R[0], R[1],
-                                                        R[2], T, accumulate ? 1 : 0);
+        smooth_kernel<T, false, false><<<grid, T::kThreads, 0, stream>>>(P, gauss_taps());
     return cudaGetLastError();
 }
 
@@ -764,30 +865,19 @@ cudaError_t launch_smooth_sparse(const int R[3], const int* table, int n_bricks,
                                  int out_stride, float empty, bool transpose, bool accumulate,
                                  cudaStream_t stream)
 {
-    SparseSmooth P;
-    P.table = table;
-    int64_t entries = 1;
-    for (int a = 0; a < 3; ++a) {
-        P.R[a] = R[a];
-        P.B[a] = R[a] / SB;
-        entries *= P.B[a];
-    }
-    P.n_bricks = n_bricks;
-    P.in = in;
-    P.in_base = in_base;
+    using T = BrickSmooth;
+    Smooth P;
+    const dim3 grid = brick_domain(R, table, n_bricks, P.D);
+    P.in = in + in_base;
     P.in_stride = in_stride;
-    P.out = out;
-    P.out_base = out_base;
+    P.out = out + out_base;
     P.out_stride = out_stride;
     P.empty = empty;
     P.accumulate = accumulate ? 1 : 0;
-    if (entries < 1 || entries > 0x7fffffff) return cudaErrorInvalidValue;
-    const Taps T = gauss_taps();
-    auto kernel = transpose ? sparse_smooth_kernel<true> : sparse_smooth_kernel<false>;
-    const cudaError_t e =
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpBytes);
-    if (e != cudaSuccess) return e;
-    kernel<<<static_cast<unsigned>(entries), kSpThreads, kSpBytes, stream>>>(P, T);
+    if (transpose)
+        smooth_kernel<T, true, true><<<grid, T::kThreads, 0, stream>>>(P, gauss_taps());
+    else
+        smooth_kernel<T, true, false><<<grid, T::kThreads, 0, stream>>>(P, gauss_taps());
     return cudaGetLastError();
 }
 
@@ -804,39 +894,15 @@ cudaError_t launch_sdf_reg(const int R[3], const float h[3], const float* s_hat,
     P.d_stride = d_stride;
     P.d_s_hat = d_s_hat;
     P.loss = loss;
-    int64_t entries = 1;
-    for (int a = 0; a < 3; ++a) {
-        P.R[a] = R[a];
-        P.inv2h[a] = 0.5f / h[a];
-        P.B[a] = R[a] / SB;
-        entries *= P.B[a];
-    }
+    for (int a = 0; a < 3; ++a) P.inv2h[a] = 0.5f / h[a];
     P.lam_sdf = lam_sdf;
     P.lam_eik = lam_eik;
     P.lam_normal = lam_normal;
-    P.table = table;
-    P.n_bricks = n_bricks;
     P.empty = empty;
     if (table) {
-        if (entries < 1 || entries > 0x7fffffff) return cudaErrorInvalidValue;
-        constexpr int kBytes = static_cast<int>(sizeof(SparseReg::Smem));
-        auto kernel = sdf_reg_kernel<SparseReg, true>;
-        cudaError_t e =
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
-        if (e != cudaSuccess) return e;
-        kernel<<<static_cast<unsigned>(entries), kRegThreads, kBytes, stream>>>(P);
-        return cudaGetLastError();
+        return launch_reg<BrickReg, true>(P, brick_domain(R, table, n_bricks, P.D), stream);
     }
-    constexpr int kBytes = static_cast<int>(sizeof(DenseReg::Smem));
-    auto kernel = sdf_reg_kernel<DenseReg, false>;
-    cudaError_t e =
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
-    if (e != cudaSuccess) return e;
-    const dim3 grid((R[0] + DenseReg::RX - 1) / DenseReg::RX,
-                    (R[1] + DenseReg::RY - 1) / DenseReg::RY,
-                    (R[2] + DenseReg::ZC - 1) / DenseReg::ZC);
-    kernel<<<grid, kRegThreads, kBytes, stream>>>(P);
-    return cudaGetLastError();
+    return launch_reg<DenseReg, false>(P, dense_domain<DenseReg>(R, 1, 6, P.D), stream);
 }
 
 cudaError_t launch_plane_reg(const float4* planes, int64_t n_texels, float lam, float4* grad,
