@@ -100,7 +100,17 @@ __global__ void occupancy_kernel(GridView g, int rx, int ry, int rz, float thres
 
 // One warp per ray: the uniform render's opacities from the SDF alone, the
 // chunk transmittance by a warp scan, per-bin sums of w_k.
-__global__ void histogram_kernel(RenderArgs A, int n_bins, float* __restrict__ hist)
+//
+// Lane l of a chunk gathers point k + 1 and takes s_k from lane l - 1 (lane 0
+// from the chunk before), so that no lane waits for a second gather after its
+// own, and the next chunk's gather is issued before this chunk's arithmetic.
+// Bound: gather latency.  Measured at 2^15 rays x 256 samples on 256^3 records:
+// 0.082 ms (0.119 ms with the second gather and no work ahead).
+constexpr int kHistWarps = 8;
+
+template <int STRIDE>
+__global__ void __launch_bounds__(32 * kHistWarps, 4) histogram_kernel(RenderArgs A, int n_bins,
+                                                                       float* __restrict__ hist)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -109,33 +119,39 @@ __global__ void histogram_kernel(RenderArgs A, int n_bins, float* __restrict__ h
     const unsigned FULL = 0xffffffffu;
     for (int64_t ray = warp0; ray < A.n_rays; ray += nwarps) {
         const RayIn R = load_ray(A, ray);
-        float o[3], d[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            o[a] = R.o[a];
-            d[a] = R.d[a];
-        }
         float tn, tf;
-        const bool hit = ray_box(o, d, A.grid, tn, tf);
+        const bool hit = ray_box(R.o, R.d, A.grid, tn, tf);
         float bins_acc = 0.0f;  // lane b < n_bins accumulates bin b
         if (hit) {
             const float dt = __fdiv_rn(__fsub_rn(tf, tn), static_cast<float>(N));
+            auto gather = [&](SdfPoint<STRIDE>& p, int k) {
+                float x[3];
+                point_at(R.o, R.d, sample_t(k < N ? k : N, dt, tn), x);
+                p.gather(A.grid, x);
+            };
+            SdfPoint<STRIDE> first, next;
+            gather(first, 0);
+            gather(next, lane + 1);
+            float s_carry = first.value(A.grid);
             float carry = 0.0f, comp = 0.0f;
             for (int base = 0; base < N; base += 32) {
+                const SdfPoint<STRIDE> cur = next;
+                if (base + 32 < N) gather(next, base + 33 + lane);
                 const int k = base + lane;
                 const bool active = k < N;
-                float x[3];
-                point_at(o, d, sample_t(active ? k : N, dt, tn), x);
-                const float s = sdf_value(A.grid, locate(x, A.grid.bmin, A.grid.sc, A.grid.R));
-                float s_next = __shfl_down_sync(FULL, s, 1);
-                if (active && (lane == 31 || k + 1 >= N)) {
-                    point_at(o, d, sample_t(k + 1, dt, tn), x);
-                    s_next = sdf_value(A.grid, locate(x, A.grid.bmin, A.grid.sc, A.grid.R));
-                }
-                float lam = 0.0f;
-                if (active) {
-                    const float diff = log_transmittance(A.tau, s, s_next);
-                    lam = diff < 0.0f ? diff : 0.0f;
+                const float s_next = cur.value(A.grid);
+                const float s = shift_up(s_next, s_carry);
+                // where the SDF does not fall the opacity is clipped to zero:
+                // without a falling sample the chunk's weights and log T are zero
+                const bool falls = active && s_next < s;
+                if (!__any_sync(FULL, falls)) continue;
+                float lam = 0.0f, alpha = 0.0f;
+                if (falls) {
+                    const float diff = log_transmittance(A.tau, s, s_next, alpha);
+                    if (diff < 0.0f)
+                        lam = diff;
+                    else
+                        alpha = 0.0f;
                 }
                 float incl = lam;
 #pragma unroll
@@ -146,7 +162,7 @@ __global__ void histogram_kernel(RenderArgs A, int n_bins, float* __restrict__ h
                 float excl = __shfl_up_sync(FULL, incl, 1);
                 if (lane == 0) excl = 0.0f;
                 const float total = __shfl_sync(FULL, incl, 31);
-                const float w = active ? expf((carry - comp) + excl) * -expm1f(lam) : 0.0f;
+                const float w = expf((carry - comp) + excl) * alpha;
                 const int my_bin = active ? k / per_bin : -1;
                 for (int b = base / per_bin; b <= min(n_bins - 1, (base + 31) / per_bin); ++b) {
                     float v = my_bin == b ? w : 0.0f;
@@ -439,42 +455,103 @@ __global__ void proposal_fwd_kernel(PropArgs P)
     }
 }
 
-__device__ __forceinline__ float warp_sum(float v)
+// Adjoint of the proposal MLP.  Threads evaluate and differentiate one ray
+// each, then the CTA sums every parameter's gradient over its 128 rays as three
+// outer products: the two factors of a layer (its inputs and its dz) are staged
+// feature by feature, and a thread owns a block of parameters whose sums stay in
+// its registers over all of its CTA's rays (two rays per paired FMA, four per
+// 16-byte read).  The layers take turns in one staging buffer.
+//
+// Bound: latency of one ray's evaluation (few warps: 2^15 rays are 1024).
+// Measured at 2^15 rays, 16 bins: 0.077 ms, against 0.504 ms with a warp sum
+// (five shuffles and a shared-memory atomic) per parameter and 32 rays.
+constexpr int kBwdThreadsP = 128;
+constexpr int kStageRow = kBwdThreadsP + 4;  // floats per feature: 16-byte rows, distinct banks
+
+template <int B>
+struct PropBwdSmem {
+    static constexpr int kIn = PropShape<B>::kIn, kInP = PropShape<B>::kInP;
+    static_assert(kPW % 16 == 0 && kIn < kInP && kInP % 8 == 0, "whole blocks of parameters");
+    float sw[PropShape<B>::kParams + 4];
+    float sw1[kPW * kInP];
+    // [dz (kPW) | inputs (layer 1: kInP, the last one 1 for the bias; layers 2
+    // and 3: kPW)] x rays
+    static constexpr int kInputs = kInP > kPW ? kInP : kPW;
+    float stage[(kPW + kInputs) * kStageRow];
+};
+
+// acc[r][c] += sum over the staged rays of dz[r0 + 16 r] x in[c0 + 8 c]
+template <int NR, int NC>
+__device__ __forceinline__ void outer_sum(const float* dz, const float* in, int r0, int c0,
+                                          float2 (&acc)[NR][NC])
 {
+#pragma unroll 2
+    for (int k = 0; k < kBwdThreadsP; k += 4) {
+        float4 a[NR], x[NC];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
+        for (int r = 0; r < NR; ++r)
+            a[r] = *reinterpret_cast<const float4*>(dz + (r0 + 16 * r) * kStageRow + k);
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            x[c] = *reinterpret_cast<const float4*>(in + (c0 + 8 * c) * kStageRow + k);
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                acc[r][c] = fma2(make_float2(a[r].x, a[r].y), make_float2(x[c].x, x[c].y),
+                                 acc[r][c]);
+                acc[r][c] = fma2(make_float2(a[r].z, a[r].w), make_float2(x[c].z, x[c].w),
+                                 acc[r][c]);
+            }
+    }
+}
+
+// Sum of a staged feature over the rays.
+__device__ __forceinline__ float2 staged_sum(const float* f, float2 acc)
+{
+    for (int k = 0; k < kBwdThreadsP; k += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(f + k);
+        acc = add2(acc, add2(make_float2(v.x, v.y), make_float2(v.z, v.w)));
+    }
+    return acc;
 }
 
 template <int B>
-__global__ void proposal_bwd_kernel(PropArgs P)
+__global__ void __launch_bounds__(kBwdThreadsP) proposal_bwd_kernel(PropArgs P)
 {
-    constexpr int kIn = PropShape<B>::kIn;
-    constexpr int kParams = PropShape<B>::kParams;
-    __shared__ __align__(16) float sw[kParams];
-    __shared__ __align__(16) float sw1[kPW * PropShape<B>::kInP];
-    __shared__ float acc[kParams];
-    extern __shared__ uint32_t sbits[];
-    load_prop_params<B>(P.params, sw, sw1);
-    for (int i = threadIdx.x; i < kParams; i += blockDim.x) acc[i] = 0.0f;
+    using M = PropBwdSmem<B>;
+    constexpr int kIn = M::kIn, kInP = M::kInP;
+    constexpr int kC1 = kInP / 8, kC2 = kPW / 8;
+    constexpr int kR3 = B / 8;  // layer 3: B rows, dz staged in the first B features
+    extern __shared__ __align__(16) uint8_t bwd_smem[];
+    M& S = *reinterpret_cast<M*>(bwd_smem);
+    uint32_t* sbits = reinterpret_cast<uint32_t*>(bwd_smem + sizeof(M));
+    load_prop_params<B>(P.params, S.sw, S.sw1);
     for (int i = threadIdx.x; i < occ_words(P); i += blockDim.x) sbits[i] = P.occ_bits[i];
     __syncthreads();
-    const float* W2 = sw + kPW * kIn + kPW;
+    const float* W2 = S.sw + kPW * kIn + kPW;
     const float* W3 = W2 + kPW * kPW + kPW;
-    float* gW1 = acc;
-    float* gb1 = gW1 + kPW * kIn;
-    float* gW2 = gb1 + kPW;
-    float* gb2 = gW2 + kPW * kPW;
-    float* gW3 = gb2 + kPW;
-    float* gb3 = gW3 + B * kPW;
-    const int lane = threadIdx.x & 31;
-    // whole warps iterate together so that the per-parameter warp sums below
-    // see every lane; lanes past the end contribute zeros
-    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-    for (int64_t base = int64_t(blockIdx.x) * blockDim.x + (threadIdx.x & ~31); base < P.n_rays;
-         base += stride) {
-        const int64_t ray = base + lane;
-        PropState<B> S;
+    float* st_dz = S.stage;
+    float* st_in = S.stage + kPW * kStageRow;
+    const int tid = threadIdx.x;
+    // this thread's block of parameters: layers 1 and 2 rows r0, r0 + 16 and
+    // columns c0, c0 + 8, ..; layer 3 rows r3 (+ 8) and columns c3 + 16 c
+    const int c0 = tid & 7, r0 = tid >> 3;
+    float2 a1[2][kC1], a2[2][kC2], a3[kR3][2], b2 = make_float2(0.f, 0.f), b3 = b2;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+        for (int c = 0; c < kC1; ++c) a1[r][c] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < kC2; ++c) a2[r][c] = make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int r = 0; r < kR3; ++r) a3[r][0] = a3[r][1] = make_float2(0.f, 0.f);
+    // CTA-uniform: lanes past the end contribute zeros
+    const int64_t stride = int64_t(gridDim.x) * kBwdThreadsP;
+    for (int64_t base = int64_t(blockIdx.x) * kBwdThreadsP; base < P.n_rays; base += stride) {
+        const int64_t ray = base + tid;
+        PropState<B> R;
         float dl[B];
         bool valid = false;
         if (ray < P.n_rays) {
@@ -484,12 +561,12 @@ __global__ void proposal_bwd_kernel(PropArgs P)
             valid = mass >= P.min_mass;
             float ce = 0.0f;
             if (valid) {
-                proposal_eval<B>(P, sw, sw1, sbits, ray, S);
+                proposal_eval<B>(P, S.sw, S.sw1, sbits, ray, R);
 #pragma unroll
                 for (int b = 0; b < B; ++b) {
                     const float h = __ldg(P.hist + ray * B + b);
-                    ce -= h * logf(S.p[b]);
-                    dl[b] = P.scale * (mass * S.p[b] - h);
+                    ce -= h * logf(R.p[b]);
+                    dl[b] = P.scale * (mass * R.p[b] - h);
                 }
             }
             if (P.loss) P.loss[ray] = ce;
@@ -498,61 +575,122 @@ __global__ void proposal_bwd_kernel(PropArgs P)
 #pragma unroll
             for (int b = 0; b < B; ++b) dl[b] = 0.0f;
 #pragma unroll
-            for (int i = 0; i < kPW; ++i) S.h1[i] = S.h2[i] = 0.0f;
+            for (int i = 0; i < kPW; ++i) R.h1[i] = R.h2[i] = 0.0f;
 #pragma unroll
-            for (int i = 0; i < kIn; ++i) S.x[i] = 0.0f;
-            S.m1 = S.m2 = 0;
+            for (int i = 0; i < kIn; ++i) R.x[i] = 0.0f;
+            R.m1 = R.m2 = 0;
         }
-        // layer 3
+        // ---- layer 3: dl (x) h2 ----
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const float sb = warp_sum(dl[b]);
-            if (lane == 0) atomicAdd(gb3 + b, sb);
-#pragma unroll 4
-            for (int i = 0; i < kPW; ++i) {
-                const float v = warp_sum(dl[b] * S.h2[i]);
-                if (lane == 0) atomicAdd(gW3 + b * kPW + i, v);
+        for (int b = 0; b < B; ++b) st_dz[b * kStageRow + tid] = dl[b];
+#pragma unroll
+        for (int i = 0; i < kPW; ++i) st_in[i * kStageRow + tid] = R.h2[i];
+        float dz[kPW];
+#pragma unroll
+        for (int i = 0; i < kPW; ++i) dz[i] = 0.0f;
+#pragma unroll
+        for (int b = 0; b < B; ++b)
+#pragma unroll
+            for (int i = 0; i < kPW; i += 4) {
+                const float4 w = *reinterpret_cast<const float4*>(W3 + b * kPW + i);
+                dz[i] = fmaf(w.x, dl[b], dz[i]);
+                dz[i + 1] = fmaf(w.y, dl[b], dz[i + 1]);
+                dz[i + 2] = fmaf(w.z, dl[b], dz[i + 2]);
+                dz[i + 3] = fmaf(w.w, dl[b], dz[i + 3]);
             }
+#pragma unroll
+        for (int i = 0; i < kPW; ++i) dz[i] = ((R.m2 >> i) & 1u) ? dz[i] : 0.0f;
+        __syncthreads();
+        {
+            // 8 row groups x 16 column groups
+            const int r3 = tid >> 4, c3 = tid & 15;
+#pragma unroll 2
+            for (int k = 0; k < kBwdThreadsP; k += 4) {
+                float4 x[2];
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    x[c] = *reinterpret_cast<const float4*>(st_in + (c3 + 16 * c) * kStageRow + k);
+#pragma unroll
+                for (int r = 0; r < kR3; ++r) {
+                    const float4 a =
+                        *reinterpret_cast<const float4*>(st_dz + (r3 + 8 * r) * kStageRow + k);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        a3[r][c] = fma2(make_float2(a.x, a.y), make_float2(x[c].x, x[c].y),
+                                        a3[r][c]);
+                        a3[r][c] = fma2(make_float2(a.z, a.w), make_float2(x[c].z, x[c].w),
+                                        a3[r][c]);
+                    }
+                }
+            }
+            if (tid < B) b3 = staged_sum(st_dz + tid * kStageRow, b3);
         }
-        float dz2[kPW];
+        __syncthreads();
+        // ---- layer 2: dz2 (x) h1 ----
 #pragma unroll
         for (int i = 0; i < kPW; ++i) {
-            float a = 0.0f;
-#pragma unroll
-            for (int b = 0; b < B; ++b) a = fmaf(W3[b * kPW + i], dl[b], a);
-            dz2[i] = ((S.m2 >> i) & 1u) ? a : 0.0f;
-        }
-#pragma unroll 4
-        for (int u = 0; u < kPW; ++u) {
-            const float sb = warp_sum(dz2[u]);
-            if (lane == 0) atomicAdd(gb2 + u, sb);
-#pragma unroll 4
-            for (int i = 0; i < kPW; ++i) {
-                const float v = warp_sum(dz2[u] * S.h1[i]);
-                if (lane == 0) atomicAdd(gW2 + u * kPW + i, v);
-            }
+            st_dz[i * kStageRow + tid] = dz[i];
+            st_in[i * kStageRow + tid] = R.h1[i];
         }
         float dz1[kPW];
 #pragma unroll
-        for (int i = 0; i < kPW; ++i) {
-            float a = 0.0f;
+        for (int i = 0; i < kPW; ++i) dz1[i] = 0.0f;
 #pragma unroll
-            for (int u = 0; u < kPW; ++u) a = fmaf(W2[u * kPW + i], dz2[u], a);
-            dz1[i] = ((S.m1 >> i) & 1u) ? a : 0.0f;
-        }
-#pragma unroll 4
-        for (int u = 0; u < kPW; ++u) {
-            const float sb = warp_sum(dz1[u]);
-            if (lane == 0) atomicAdd(gb1 + u, sb);
+        for (int u = 0; u < kPW; ++u)
 #pragma unroll
-            for (int i = 0; i < kIn; ++i) {
-                const float v = warp_sum(dz1[u] * S.x[i]);
-                if (lane == 0) atomicAdd(gW1 + u * kIn + i, v);
+            for (int i = 0; i < kPW; i += 4) {
+                const float4 w = *reinterpret_cast<const float4*>(W2 + u * kPW + i);
+                dz1[i] = fmaf(w.x, dz[u], dz1[i]);
+                dz1[i + 1] = fmaf(w.y, dz[u], dz1[i + 1]);
+                dz1[i + 2] = fmaf(w.z, dz[u], dz1[i + 2]);
+                dz1[i + 3] = fmaf(w.w, dz[u], dz1[i + 3]);
             }
-        }
+#pragma unroll
+        for (int i = 0; i < kPW; ++i) dz1[i] = ((R.m1 >> i) & 1u) ? dz1[i] : 0.0f;
+        __syncthreads();
+        outer_sum(st_dz, st_in, r0, c0, a2);
+        if (tid < kPW) b2 = staged_sum(st_dz + tid * kStageRow, b2);
+        __syncthreads();
+        // ---- layer 1: dz1 (x) [x, 1] ----
+#pragma unroll
+        for (int i = 0; i < kPW; ++i) st_dz[i * kStageRow + tid] = dz1[i];
+#pragma unroll
+        for (int i = 0; i < kInP; ++i)
+            st_in[i * kStageRow + tid] = i < kIn ? R.x[i] : (i == kIn ? 1.0f : 0.0f);
+        __syncthreads();
+        outer_sum(st_dz, st_in, r0, c0, a1);
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kParams; i += blockDim.x) red_add(P.grad + i, acc[i]);
+    float* gW1 = P.grad;
+    float* gb1 = gW1 + kPW * kIn;
+    float* gW2 = gb1 + kPW;
+    float* gb2 = gW2 + kPW * kPW;
+    float* gW3 = gb2 + kPW;
+    float* gb3 = gW3 + B * kPW;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int u = r0 + 16 * r;
+#pragma unroll
+        for (int c = 0; c < kC1; ++c) {
+            const int i = c0 + 8 * c;
+            const float v = a1[r][c].x + a1[r][c].y;
+            if (i < kIn)
+                red_add(gW1 + u * kIn + i, v);
+            else if (i == kIn)
+                red_add(gb1 + u, v);
+        }
+#pragma unroll
+        for (int c = 0; c < kC2; ++c)
+            red_add(gW2 + u * kPW + c0 + 8 * c, a2[r][c].x + a2[r][c].y);
+    }
+#pragma unroll
+    for (int r = 0; r < kR3; ++r)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            red_add(gW3 + ((tid >> 4) + 8 * r) * kPW + (tid & 15) + 16 * c,
+                    a3[r][c].x + a3[r][c].y);
+    if (tid < kPW) red_add(gb2 + tid, b2.x + b2.y);
+    if (tid < B) red_add(gb3 + tid, b3.x + b3.y);
 }
 
 int blocks_for(int64_t n, int threads, int cap)
@@ -595,9 +733,11 @@ cudaError_t launch_occupancy(const GridView& g, const int res[3], float threshol
 
 cudaError_t launch_histogram(const RenderArgs& A, int n_bins, float* hist, cudaStream_t stream)
 {
-    const int64_t warps = A.n_rays;
-    histogram_kernel<<<blocks_for(warps * 32, 256, 16 * sm_count()), 256, 0, stream>>>(
-        A, n_bins, hist);
+    const int blocks = blocks_for(A.n_rays * 32, 32 * kHistWarps, 16 * sm_count());
+    auto kernel = A.grid.table ? histogram_kernel<0>
+                  : A.grid.sdf ? histogram_kernel<1>
+                               : histogram_kernel<4>;
+    kernel<<<blocks, 32 * kHistWarps, 0, stream>>>(A, n_bins, hist);
     return cudaGetLastError();
 }
 
@@ -649,10 +789,12 @@ cudaError_t launch_fwd(const PropArgs& P, cudaStream_t stream)
 template <int B>
 cudaError_t launch_bwd(const PropArgs& P, cudaStream_t stream)
 {
-    const size_t smem = sizeof(uint32_t) * occupancy_words(P.occ_res);
+    const size_t smem = sizeof(PropBwdSmem<B>) + sizeof(uint32_t) * occupancy_words(P.occ_res);
     cudaError_t e = allow_smem(proposal_bwd_kernel<B>, smem);
     if (e != cudaSuccess) return e;
-    proposal_bwd_kernel<B><<<blocks_for(P.n_rays, 128, 4 * sm_count()), 128, smem, stream>>>(P);
+    // 2 CTAs per SM fit with the largest bitmask (registers and shared memory)
+    proposal_bwd_kernel<B><<<blocks_for(P.n_rays, kBwdThreadsP, 2 * sm_count()), kBwdThreadsP,
+                             smem, stream>>>(P);
     return cudaGetLastError();
 }
 

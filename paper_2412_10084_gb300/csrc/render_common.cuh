@@ -438,6 +438,56 @@ __device__ __forceinline__ float sdf_value(const GridView& g, const Cell& c)
     return sdf_corners_combine(c, v);
 }
 
+// SDF of a point in two halves, the gather and the interpolation, so that a march
+// can have the next points' gathers in flight while it works on the current ones.
+// The value has the bits of sdf_value.  STRIDE: floats between the SDF values of
+// x-neighbours (4 in FP32 node records, 1 in an array of their own); 0: sparse.
+template <int STRIDE>
+struct SdfPoint {
+    Cell c;
+    float v[8];
+    bool empty;  // sparse: no corner is stored
+    __device__ __forceinline__ void gather(const GridView& g, const float x[3])
+    {
+        c = locate(x, g.bmin, g.sc, g.R);
+        empty = false;
+        if constexpr (STRIDE == 0) {
+            int64_t rec[8];
+            empty = brick_corners(g, c.i, rec) == 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                v[q] = rec[q] >= 0 ? __ldg(reinterpret_cast<const float*>(g.nodes + rec[q]))
+                                   : g.empty_sdf;
+        } else {
+            const float* base = STRIDE == 1 ? g.sdf : reinterpret_cast<const float*>(g.nodes);
+            const int64_t sy = int64_t(STRIDE) * g.R[0], sz = sy * g.R[1];
+            const float* p[4];
+            p[0] = base + int64_t(STRIDE) * c.base;
+            p[1] = p[0] + sy;
+            p[2] = p[0] + sz;
+            p[3] = p[1] + sz;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = __ldg(p[q >> 1] + STRIDE * (q & 1));
+        }
+    }
+    __device__ __forceinline__ float value(const GridView& g) const
+    {
+        return STRIDE == 0 && empty ? g.empty_sdf : sdf_corners_combine(c, v);
+    }
+};
+
+// The lane below's value, lane 0 taking lane 31's of the call before (`carry`,
+// kept by lane 0; the other lanes' carries are unused).
+template <class V>
+__device__ __forceinline__ V shift_up(V v, V& carry)
+{
+    const int lane = threadIdx.x & 31;
+    const V x = __shfl_sync(0xffffffffu, v, (lane + 31) & 31);
+    const V r = lane == 0 ? carry : x;
+    carry = x;
+    return r;
+}
+
 // Value, analytic gradient (world units) and 3 features at a point.
 __device__ __forceinline__ void sdf_full(const GridView& g, const Cell& c, const Corners& k,
                                          float& s, float grad[3], float feat[3])
@@ -561,6 +611,20 @@ __device__ __forceinline__ float log_transmittance(float tau, float s0, float s1
     const float p = expm1f(tau * (s1 - s0)) / (1.0f + expf(tau * s1));
     if (p > -0.5f) return log1pf(p);
     return log_phi(tau, s1) - log_phi(tau, s0);
+}
+
+// log_transmittance with the opacity itself: alpha = 1 - (1 - alpha) = -p where
+// the logarithm is log1p(p), which saves its expm1 and a rounding.
+__device__ __forceinline__ float log_transmittance(float tau, float s0, float s1, float& alpha)
+{
+    const float p = expm1f(tau * (s1 - s0)) / (1.0f + expf(tau * s1));
+    if (p > -0.5f) {
+        alpha = -p;
+        return log1pf(p);
+    }
+    const float d = log_phi(tau, s1) - log_phi(tau, s0);
+    alpha = -expm1f(d);
+    return d;
 }
 
 // d log Phi / ds = tau * (1 - Phi(s)) = tau * sigmoid(-tau s)
