@@ -258,17 +258,35 @@ done:
 
 constexpr int kRenderWarps = 8;
 
-__global__ void __launch_bounds__(kRenderWarps * 32) colour_render_kernel(
+// Lane l of a chunk gathers point k + 1's SDF and takes sample k's distance, SDF
+// and cell from lane l - 1 (lane 0 from the chunk before), so that no lane waits
+// for a second gather after its own; a chunk in which the SDF falls nowhere ends
+// there (its weights are zero); a CTA's warps take its rays from a counter (a ray
+// that misses the box costs next to nothing).
+//
+// Bound: issue (65-70 %; the logarithms of the opacity) and gather latency.
+// 32 warps per SM at 64 registers.  Measured on a 1080p view, 256 samples: 1.9-2.2
+// ms by view, against 2.86 ms with 24 warps and a second gather per chunk; with
+// the next chunk's gather issued ahead the spills cost 0.2 ms.
+template <int STRIDE>
+__global__ void __launch_bounds__(kRenderWarps * 32, 4) colour_render_kernel(
     RenderArgs A, const uint2* __restrict__ colours)
 {
     __shared__ float tab[kRenderWarps][64];
+    __shared__ int counter;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     const int N = A.n_samples;
-    const int sx = 1, sy = A.grid.R[0], sz = A.grid.R[0] * A.grid.R[1];
-    const int off[8] = {0, sx, sy, sx + sy, sz, sz + sx, sz + sy, sz + sy + sx};
     const int64_t stride = int64_t(gridDim.x) * kRenderWarps;
-    for (int64_t ray = int64_t(blockIdx.x) * kRenderWarps + warp; ray < A.n_rays; ray += stride) {
+    if (threadIdx.x == 0) counter = 0;
+    __syncthreads();
+    for (;;) {
+        int j = 0;
+        if (lane == 0) j = atomicAdd(&counter, 1);
+        j = __shfl_sync(FULL, j, 0);
+        const int64_t ray = int64_t(blockIdx.x) * kRenderWarps + j % kRenderWarps +
+                            int64_t(j / kRenderWarps) * stride;
+        if (ray >= A.n_rays) break;  // later ones are past the end too
         const RayIn R = load_ray(A, ray);
         const RaySpan sp = ray_span(A, R, ray, tab[warp]);
         if (!sp.hit) {
@@ -281,34 +299,54 @@ __global__ void __launch_bounds__(kRenderWarps * 32) colour_render_kernel(
             }
             continue;
         }
+        auto gather = [&](SdfPoint<STRIDE>& p, int k) {
+            const float t = span_t(sp, k < N ? k : N);
+            float x[3];
+            point_at(R.o, R.d, t, x);
+            p.gather(A.grid, x);
+            return t;
+        };
+        SdfPoint<STRIDE> first;
+        float t_carry = gather(first, 0);
+        float s_carry = first.value(A.grid);
+        Cell c_carry = first.c;
         float acc_r = 0.f, acc_g = 0.f, acc_b = 0.f, acc_d = 0.f, acc_w = 0.f;
         float carry = 0.f, comp = 0.f;  // Kahan sum of log T over chunks
         for (int base = 0; base < N; base += 32) {
             const int k = base + lane;
             const bool active = k < N;
-            const float t = span_t(sp, active ? k : N - 1);
-            float xw[3];
-            point_at(R.o, R.d, t, xw);
-            const Cell cell = locate(xw, A.grid.bmin, A.grid.sc, A.grid.R);
-            const float s = sdf_value(A.grid, cell);
-            float s_next = __shfl_down_sync(FULL, s, 1);
-            if (active && (lane == 31 || k + 1 >= N)) {
-                float xn[3];
-                point_at(R.o, R.d, span_t(sp, k + 1), xn);
-                s_next = sdf_value(A.grid, locate(xn, A.grid.bmin, A.grid.sc, A.grid.R));
-            }
-            float lam = 0.0f;
-            if (active) {
-                const float diff = log_transmittance(A.tau, s, s_next);
-                lam = diff < 0.0f ? diff : 0.0f;
+            SdfPoint<STRIDE> cur;
+            const float t1 = gather(cur, k + 1);
+            const float s1 = cur.value(A.grid);
+            const float t = shift_up(t1, t_carry), s = shift_up(s1, s_carry);
+            // sample k's cell is the one lane l - 1 gathered
+            Cell cell;
+            cell.base = shift_up(cur.c.base, c_carry.base);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) cell.f[a] = shift_up(cur.c.f[a], c_carry.f[a]);
+            // where the SDF does not fall the opacity is clipped to zero
+            const bool falls = active && s1 < s;
+            if (!__any_sync(FULL, falls)) continue;
+            float lam = 0.0f, alpha = 0.0f;
+            if (falls) {
+                const float diff = log_transmittance(A.tau, s, s1, alpha);
+                if (diff < 0.0f)
+                    lam = diff;
+                else
+                    alpha = 0.0f;
             }
             float cr = 0.f, cg = 0.f, cb = 0.f;
             if (lam < 0.0f) {  // alpha > 0: the colour reaches the outputs
                 float w[8];
                 corner_weights(cell.f, w);
+                const uint2* p[4];
+                p[0] = colours + cell.base;
+                p[1] = p[0] + A.grid.R[0];
+                p[2] = p[0] + int64_t(A.grid.R[0]) * A.grid.R[1];
+                p[3] = p[2] + A.grid.R[0];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                    const uint2 u = __ldg(colours + cell.base + off[q]);
+                    const uint2 u = __ldg(p[q >> 1] + (q & 1));
                     const float2 rg = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
                     const float2 b0 = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
                     cr = fmaf(w[q], rg.x, cr);
@@ -326,7 +364,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32) colour_render_kernel(
             float excl = __shfl_up_sync(FULL, incl, 1);
             if (lane == 0) excl = 0.0f;
             const float total = __shfl_sync(FULL, incl, 31);
-            const float wgt = active ? expf((carry - comp) + excl) * -expm1f(lam) : 0.0f;
+            const float wgt = expf((carry - comp) + excl) * alpha;
             {
                 const float y = total - comp;
                 const float tt = carry + y;
@@ -336,7 +374,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32) colour_render_kernel(
             acc_r = fmaf(wgt, cr, acc_r);
             acc_g = fmaf(wgt, cg, acc_g);
             acc_b = fmaf(wgt, cb, acc_b);
-            acc_d = fmaf(wgt, t, acc_d);
+            if (active) acc_d = fmaf(wgt, t, acc_d);
             acc_w += wgt;
         }
 #pragma unroll
@@ -402,15 +440,17 @@ cudaError_t launch_colour_render(const RenderArgs& A, const void* colours, cudaS
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    auto kernel = A.grid.table ? colour_render_kernel<0>
+                  : A.grid.sdf ? colour_render_kernel<1>
+                               : colour_render_kernel<4>;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, colour_render_kernel,
-                                                                  kRenderWarps * 32, 0);
+    cudaError_t e =
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRenderWarps * 32, 0);
     if (e != cudaSuccess) return e;
     const int64_t need = (A.n_rays + kRenderWarps - 1) / kRenderWarps;
     const int64_t full = int64_t(sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
     const int ctas = static_cast<int>(need < full ? need : full);
-    colour_render_kernel<<<ctas, kRenderWarps * 32, 0, stream>>>(
-        A, static_cast<const uint2*>(colours));
+    kernel<<<ctas, kRenderWarps * 32, 0, stream>>>(A, static_cast<const uint2*>(colours));
     return cudaGetLastError();
 }
 
