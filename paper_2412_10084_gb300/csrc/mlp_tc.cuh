@@ -36,9 +36,12 @@ struct MlpTC {
 
 // Cooperative load of the packed FP32 parameters into the split weight tiles
 // (hi at w, lo at w + kW1 / + kW2) and the FP32 block.
-template <class C>
+// BIAS1: b1 goes into the columns NIN (its FP16 part) and NIN + 1 (the rest) of
+// W1's hi tile, for input rows that hold 1 in both.
+template <class C, bool BIAS1 = false>
 __device__ __forceinline__ void load_mlp_tc(const float* __restrict__ g, uint8_t* wt, float* f32)
 {
+    static_assert(C::NIN + 2 <= MlpTC<C>::K1, "two bias columns");
     using M = MlpTC<C>;
     constexpr int W = C::W;
     uint8_t* w1h = M::w1h(wt);
@@ -50,6 +53,11 @@ __device__ __forceinline__ void load_mlp_tc(const float* __restrict__ g, uint8_t
         const float v = j < C::NIN ? g[C::gW1 + o * C::NIN + j] : 0.0f;
         __half h, l;
         tc::split2(v, h, l);
+        if (BIAS1 && (j == C::NIN || j == C::NIN + 1)) {
+            tc::split2(g[C::gB1 + o], h, l);
+            if (j == C::NIN + 1) h = l;
+            l = __float2half_rn(0.0f);
+        }
         const uint32_t off = tc::tile_off(o, j, M::K1);
         *reinterpret_cast<__half*>(w1h + off) = h;
         if constexpr (M::kSplit == 2) *reinterpret_cast<__half*>(w1l + off) = l;
@@ -106,26 +114,38 @@ __device__ __forceinline__ void mma_k(uint32_t d, const uint8_t* a_hi, const uin
     }
 }
 
-// Layer 3 (W -> 3) and the sigmoid on the CUDA cores: h2 already ReLU'd.
+// Layer 3 (W -> 3) and the sigmoid on the CUDA cores, h2 already ReLU'd and
+// given part by part: even and odd hidden units summed apart, one paired FMA
+// per output and pair.
 template <class C>
-__device__ __forceinline__ void mlp_layer3(const float* f32, const float* h2, float col[3])
-{
+struct Layer3 {
     using M = MlpTC<C>;
-    constexpr int W = C::W;
-    const float4 b3 = *reinterpret_cast<const float4*>(f32 + M::kB3);
-    // even and odd hidden units summed apart, one paired FMA per output and pair
-    float2 z0 = make_float2(0.0f, 0.0f), z1 = z0, z2 = z0;
+    float2 z0 = {0.0f, 0.0f}, z1 = {0.0f, 0.0f}, z2 = {0.0f, 0.0f};
+    // units [u0, u0 + NV)
+    template <int NV>
+    __device__ __forceinline__ void add(const float* f32, int u0, const float* h2)
+    {
+        constexpr int W = C::W;
+        const float* w = f32 + M::kW3 + u0;
 #pragma unroll
-    for (int o = 0; o < W; o += 2) {
-        const float2 h = make_float2(h2[o], h2[o + 1]);
-        z0 = fma2(*reinterpret_cast<const float2*>(f32 + M::kW3 + o), h, z0);
-        z1 = fma2(*reinterpret_cast<const float2*>(f32 + M::kW3 + W + o), h, z1);
-        z2 = fma2(*reinterpret_cast<const float2*>(f32 + M::kW3 + 2 * W + o), h, z2);
+        for (int o = 0; o < NV; o += 4) {
+            const float2 ha = make_float2(h2[o], h2[o + 1]), hb = make_float2(h2[o + 2], h2[o + 3]);
+            const float4 w0 = *reinterpret_cast<const float4*>(w + o);
+            const float4 w1 = *reinterpret_cast<const float4*>(w + W + o);
+            const float4 w2 = *reinterpret_cast<const float4*>(w + 2 * W + o);
+            z0 = fma2(make_float2(w0.z, w0.w), hb, fma2(make_float2(w0.x, w0.y), ha, z0));
+            z1 = fma2(make_float2(w1.z, w1.w), hb, fma2(make_float2(w1.x, w1.y), ha, z1));
+            z2 = fma2(make_float2(w2.z, w2.w), hb, fma2(make_float2(w2.x, w2.y), ha, z2));
+        }
     }
-    col[0] = sigmoidf(b3.x + (z0.x + z0.y));
-    col[1] = sigmoidf(b3.y + (z1.x + z1.y));
-    col[2] = sigmoidf(b3.z + (z2.x + z2.y));
-}
+    __device__ __forceinline__ void colour(const float* f32, float col[3]) const
+    {
+        const float4 b3 = *reinterpret_cast<const float4*>(f32 + M::kB3);
+        col[0] = sigmoidf(b3.x + (z0.x + z0.y));
+        col[1] = sigmoidf(b3.y + (z1.x + z1.y));
+        col[2] = sigmoidf(b3.z + (z2.x + z2.y));
+    }
+};
 
 // z = max(z + b, 0) over a row of NV hidden units (bias added in pairs).
 template <int NV>
@@ -137,6 +157,14 @@ __device__ __forceinline__ void bias_relu(float* z, const float* b)
         z[o] = fmaxf(h.x, 0.0f);
         z[o + 1] = fmaxf(h.y, 0.0f);
     }
+}
+
+// z = max(z, 0): the bias is already in the accumulator.
+template <int NV>
+__device__ __forceinline__ void relu(float* z)
+{
+#pragma unroll
+    for (int o = 0; o < NV; ++o) z[o] = fmaxf(z[o], 0.0f);
 }
 
 // bias_relu that also returns the mask of the units with z + b > 0.

@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(32 * kHistWarps, 4) histogram_kernel(RenderArg
                 if (!__any_sync(FULL, falls)) continue;
                 float lam = 0.0f, alpha = 0.0f;
                 if (falls) {
-                    const float diff = log_transmittance(A.tau, s, s_next, alpha);
+                    const float diff = log_transmittance(A.tau, s, s_next, expf(A.tau * s_next), alpha);
                     if (diff < 0.0f)
                         lam = diff;
                     else

@@ -384,7 +384,9 @@ render_backward_kernel(RenderArgs A)
                 }
                 s_first = __shfl_sync(FULL, S.s, 0);
                 if (active) {
-                    const float diff = log_transmittance(tau, S.s, s_next);
+                    float alpha_p;  // the adjoint takes alpha from lam
+                    const float diff =
+                        log_transmittance(tau, S.s, s_next, expf(tau * s_next), alpha_p);
                     unclipped = diff < 0.0f;
                     lam = unclipped ? diff : 0.0f;
                 }
@@ -479,7 +481,9 @@ render_backward_kernel(RenderArgs A)
             {
                 tc::tmem_ld<W>(t_row + 32, h2);
                 mask2 = bias_relu_mask<W>(h2, f32 + M::kB2);
-                mlp_layer3<C>(f32, h2, col);
+                Layer3<C> l3;
+                l3.template add<W>(f32, 0, h2);
+                l3.colour(f32, col);
             }
             const float w = active ? Tk * alpha : 0.0f;
             const float G = active ? drgb[0] * col[0] + drgb[1] * col[1] + drgb[2] * col[2] +
@@ -507,7 +511,7 @@ render_backward_kernel(RenderArgs A)
             const float dlam = unclipped ? -Tk1 * (G - Shat) : 0.0f;
             float dlam_prev = __shfl_up_sync(FULL, dlam, 1);
             if (lane == 0) dlam_prev = 0.0f;
-            const float ds_own = active ? (dlam_prev - dlam) * dlog_phi(tau, S.s) : 0.0f;
+            const float ds_own = active ? (dlam_prev - dlam) * dlog_phi(tau, expf(tau * S.s)) : 0.0f;
 
             float dz3[3];
 #pragma unroll
@@ -783,7 +787,7 @@ render_backward_kernel(RenderArgs A)
                     }
                 }
                 if (extra) {
-                    const float ds1 = dlam * dlog_phi(tau, s_next);
+                    const float ds1 = dlam * dlog_phi(tau, expf(tau * s_next));
                     if (ds1 != 0.0f) {
                         float w1[8];
                         corner_weights(c1.f, w1);

@@ -279,6 +279,13 @@ __device__ __forceinline__ void corner_weights(const float f[3], float w[8])
     w[7] = x1 * y1 * z1;
 }
 
+// corner_weights one corner at a time (the same bits).
+__device__ __forceinline__ float corner_weight(const float f[3], int q)
+{
+    return ((q & 1) ? f[0] : 1.0f - f[0]) * ((q & 2) ? f[1] : 1.0f - f[1]) *
+           ((q & 4) ? f[2] : 1.0f - f[2]);
+}
+
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
 
@@ -450,6 +457,10 @@ struct SdfPoint {
     __device__ __forceinline__ void gather(const GridView& g, const float x[3])
     {
         c = locate(x, g.bmin, g.sc, g.R);
+        gather_cell(g);
+    }
+    __device__ __forceinline__ void gather_cell(const GridView& g)
+    {
         empty = false;
         if constexpr (STRIDE == 0) {
             int64_t rec[8];
@@ -606,18 +617,12 @@ __device__ __forceinline__ float log_phi(float tau, float s)
 // where the difference of the two logarithms cancels in FP32.  When the
 // argument nears -1 (a large drop deep inside the surface) the plain
 // difference is already accurate and avoids log1p(-1).
-__device__ __forceinline__ float log_transmittance(float tau, float s0, float s1)
+// e1 is exp(tau s1).  The opacity itself comes along: alpha = 1 - (1 - alpha) =
+// -p where the logarithm is log1p(p), which saves its expm1 and a rounding.
+__device__ __forceinline__ float log_transmittance(float tau, float s0, float s1, float e1,
+                                                   float& alpha)
 {
-    const float p = expm1f(tau * (s1 - s0)) / (1.0f + expf(tau * s1));
-    if (p > -0.5f) return log1pf(p);
-    return log_phi(tau, s1) - log_phi(tau, s0);
-}
-
-// log_transmittance with the opacity itself: alpha = 1 - (1 - alpha) = -p where
-// the logarithm is log1p(p), which saves its expm1 and a rounding.
-__device__ __forceinline__ float log_transmittance(float tau, float s0, float s1, float& alpha)
-{
-    const float p = expm1f(tau * (s1 - s0)) / (1.0f + expf(tau * s1));
+    const float p = expm1f(tau * (s1 - s0)) / (1.0f + e1);
     if (p > -0.5f) {
         alpha = -p;
         return log1pf(p);
@@ -627,11 +632,17 @@ __device__ __forceinline__ float log_transmittance(float tau, float s0, float s1
     return d;
 }
 
-// d log Phi / ds = tau * (1 - Phi(s)) = tau * sigmoid(-tau s)
-__device__ __forceinline__ float dlog_phi(float tau, float s)
+// sum += v, compensated: the sum is `sum - comp`.
+__device__ __forceinline__ void kahan_add(float& sum, float& comp, float v)
 {
-    return tau / (1.0f + expf(tau * s));
+    const float y = v - comp;
+    const float t = sum + y;
+    comp = (t - sum) - y;
+    sum = t;
 }
+
+// d log Phi / ds = tau * (1 - Phi(s)) = tau * sigmoid(-tau s), from e = exp(tau s)
+__device__ __forceinline__ float dlog_phi(float tau, float e) { return tau / (1.0f + e); }
 
 __device__ __forceinline__ float sigmoidf(float z) { return 1.0f / (1.0f + expf(-z)); }
 

@@ -100,6 +100,37 @@ __device__ __forceinline__ void probe_corner_index(const ProbeView& p, const Cel
     idx[7] = pc.base + sz + sy + sx;
 }
 
+// Blended probe coefficients b^_j = sum_i w_i b_ij (Eq. 7 before the SH
+// contraction), two channels per element, the probes in corner order.
+template <class C>
+__device__ __forceinline__ void blend_probes(const ProbeView& p, const Cell& pc, float2* B2)
+{
+#pragma unroll
+    for (int i = 0; i < C::L2 * C::NA / 2; ++i) B2[i] = make_float2(0.0f, 0.0f);
+    const float x1 = pc.f[0], x0 = 1.0f - x1;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const float y = (r & 1) ? pc.f[1] : 1.0f - pc.f[1];
+        const float z = (r & 2) ? pc.f[2] : 1.0f - pc.f[2];
+        const int row = pc.base + ((r & 1) ? p.P[0] : 0) + ((r & 2) ? p.P[0] * p.P[1] : 0);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const float w = (q ? x1 : x0) * y * z;  // as corner_weights
+            const float2 w2 = make_float2(w, w);
+#pragma unroll
+            for (int j = 0; j < C::L2; ++j) {
+#pragma unroll
+                for (int cg = 0; cg < C::NA4; ++cg) {
+                    const float4 bb = probe_coeffs<C>(p, row + q, j, cg);
+                    float2* b2 = B2 + (j * C::NA + 4 * cg) / 2;
+                    b2[0] = fma2(w2, make_float2(bb.x, bb.y), b2[0]);
+                    b2[1] = fma2(w2, make_float2(bb.z, bb.w), b2[1]);
+                }
+            }
+        }
+    }
+}
+
 // SDF part of a sample: cell, trilinear SDF value and gradient, spatial
 // features (MLP input columns 0..2).
 template <class C>
@@ -213,33 +244,14 @@ __device__ __forceinline__ void eval_appearance_at(const RenderArgs& A, const fl
 
     // Angular features (Eqs. 6-7): F_a = sum_i w_i sum_j b_ij Y_j(r).
     S.pcell = locate(xw, A.grid.bmin, A.probes.sc, A.probes.P);
-    float wq[8];
-    corner_weights(S.pcell.f, wq);
-    int pidx[8];
-    probe_corner_index(A.probes, S.pcell, pidx);
     float2 fa[C::NA / 2];
 #pragma unroll
     for (int c = 0; c < C::NA / 2; ++c) fa[c] = make_float2(0.0f, 0.0f);
     if constexpr (C::L2 * C::NA <= 36) {
-        // blended coefficients b^_j = sum_i w_i b_ij first (one weight per
-        // probe serves all of its coefficients), then F_a = sum_j Y_j b^_j
+        // blended coefficients first (one weight per probe serves all of its
+        // coefficients), then F_a = sum_j Y_j b^_j
         float2 B2[C::L2 * C::NA / 2];
-#pragma unroll
-        for (int i = 0; i < C::L2 * C::NA / 2; ++i) B2[i] = make_float2(0.0f, 0.0f);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float2 w2 = make_float2(wq[q], wq[q]);
-#pragma unroll
-            for (int j = 0; j < C::L2; ++j) {
-#pragma unroll
-                for (int cg = 0; cg < C::NA4; ++cg) {
-                    const float4 bb = probe_coeffs<C>(A.probes, pidx[q], j, cg);
-                    float2* b2 = B2 + (j * C::NA + 4 * cg) / 2;
-                    b2[0] = fma2(w2, make_float2(bb.x, bb.y), b2[0]);
-                    b2[1] = fma2(w2, make_float2(bb.z, bb.w), b2[1]);
-                }
-            }
-        }
+        blend_probes<C>(A.probes, S.pcell, B2);
 #pragma unroll
         for (int j = 0; j < C::L2; ++j) {
             const float2 y = make_float2(S.Y[j], S.Y[j]);
@@ -249,8 +261,13 @@ __device__ __forceinline__ void eval_appearance_at(const RenderArgs& A, const fl
     } else {
         // wide rows (more SH coefficients or channels): one probe at a time,
         // F_a += w_i sum_j b_ij Y_j, so only NA partial sums are live
+        const float x1 = S.pcell.f[0], x0 = 1.0f - x1;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
+            const float wq = ((q & 1) ? x1 : x0) * ((q & 2) ? S.pcell.f[1] : 1.0f - S.pcell.f[1]) *
+                             ((q & 4) ? S.pcell.f[2] : 1.0f - S.pcell.f[2]);
+            const int probe = S.pcell.base + (q & 1) + ((q & 2) ? A.probes.P[0] : 0) +
+                              ((q & 4) ? A.probes.P[0] * A.probes.P[1] : 0);
             float2 part[C::NA / 2];
 #pragma unroll
             for (int c = 0; c < C::NA / 2; ++c) part[c] = make_float2(0.0f, 0.0f);
@@ -259,12 +276,12 @@ __device__ __forceinline__ void eval_appearance_at(const RenderArgs& A, const fl
                 const float2 y = make_float2(S.Y[j], S.Y[j]);
 #pragma unroll
                 for (int cg = 0; cg < C::NA4; ++cg) {
-                    const float4 bb = probe_coeffs<C>(A.probes, pidx[q], j, cg);
+                    const float4 bb = probe_coeffs<C>(A.probes, probe, j, cg);
                     part[2 * cg] = fma2(make_float2(bb.x, bb.y), y, part[2 * cg]);
                     part[2 * cg + 1] = fma2(make_float2(bb.z, bb.w), y, part[2 * cg + 1]);
                 }
             }
-            const float2 w2 = make_float2(wq[q], wq[q]);
+            const float2 w2 = make_float2(wq, wq);
 #pragma unroll
             for (int c = 0; c < C::NA / 2; ++c) fa[c] = fma2(w2, part[c], fa[c]);
         }
@@ -325,28 +342,8 @@ __device__ __forceinline__ void eval_appearance_blend(const RenderArgs& A, const
     float xw[3];
     point_at(o, d, t, xw);
     S.pcell = locate(xw, A.grid.bmin, A.probes.sc, A.probes.P);
-    float wq[8];
-    corner_weights(S.pcell.f, wq);
-    int pidx[8];
-    probe_corner_index(A.probes, S.pcell, pidx);
-    // channel pairs of every coefficient accumulated as float2 (paired FMAs)
     float2 B2[C::L2 * C::NA / 2];
-#pragma unroll
-    for (int i = 0; i < C::L2 * C::NA / 2; ++i) B2[i] = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const float2 w2 = make_float2(wq[q], wq[q]);
-#pragma unroll
-        for (int j = 0; j < C::L2; ++j) {
-#pragma unroll
-            for (int cg = 0; cg < C::NA4; ++cg) {
-                const float4 bb = probe_coeffs<C>(A.probes, pidx[q], j, cg);
-                float2* b2 = B2 + (j * C::NA + 4 * cg) / 2;
-                b2[0] = fma2(w2, make_float2(bb.x, bb.y), b2[0]);
-                b2[1] = fma2(w2, make_float2(bb.z, bb.w), b2[1]);
-            }
-        }
-    }
+    blend_probes<C>(A.probes, S.pcell, B2);
 #pragma unroll
     for (int i = 0; i < C::L2 * C::NA / 2; ++i) {
         Bc[2 * i] = B2[i].x;
@@ -417,6 +414,23 @@ struct RaySpan {
     const float* tab;
 };
 
+// Running sums and reciprocals of a ray's bin densities into the warp's table
+// (out of line, so that the other modes' loops do not carry its code).
+static __device__ __noinline__ void bin_table(const float* q_ray, int n_bins, float* tab)
+{
+    const int lane = threadIdx.x & 31;
+    const float q = lane < n_bins ? __ldg(q_ray + lane) : 0.0f;
+    float c = 0.0f;
+    for (int i = 0; i < n_bins; ++i) {  // running sums in bin order
+        const float qi = __shfl_sync(0xffffffffu, q, i);
+        if (i < lane) c += qi;
+    }
+    __syncwarp();  // the previous ray's readers are done with the table
+    tab[lane] = c;
+    tab[32 + lane] = lane < n_bins ? 1.0f / q : 0.0f;
+    __syncwarp();
+}
+
 // tab: this warp's 64-float shared-memory table (used in the bin-density
 // mode).  Warp-uniform: every lane of the warp calls it for the warp's ray.
 __device__ __forceinline__ RaySpan ray_span(const RenderArgs& A, const RayIn& R, int64_t ray,
@@ -431,34 +445,20 @@ __device__ __forceinline__ RaySpan ray_span(const RenderArgs& A, const RayIn& R,
     sp.n = A.n_samples;
     sp.inv_n = 0.0f;
     sp.tab = tab;
-    if (A.t_samples && A.n_bins > 0) {
-        const int lane = threadIdx.x & 31;
-        float tf;
-        sp.hit = ray_box(R.o, R.d, A.grid, sp.tn, tf);
-        sp.tf = tf;
-        sp.n_bins = A.n_bins;
-        const float q = lane < A.n_bins ? __ldg(A.t_samples + ray * (int64_t)A.n_bins + lane) : 0.0f;
-        float c = 0.0f;
-        for (int i = 0; i < A.n_bins; ++i) {  // running sums in bin order
-            const float qi = __shfl_sync(0xffffffffu, q, i);
-            if (i < lane) c += qi;
-        }
-        __syncwarp();  // the previous ray's readers are done with the table
-        tab[lane] = c;
-        tab[32 + lane] = lane < A.n_bins ? 1.0f / q : 0.0f;
-        __syncwarp();
-        sp.dt = (tf - sp.tn) / A.n_bins;
-        sp.inv_n = 1.0f / A.n_samples;
-        return sp;
-    }
-    if (A.t_samples) {
+    if (A.t_samples && A.n_bins == 0) {
         sp.tk = A.t_samples + ray * (int64_t)(A.n_samples + 1);
         sp.hit = __ldg(sp.tk + A.n_samples) > __ldg(sp.tk);
         return sp;
     }
-    float tf;
-    sp.hit = ray_box(R.o, R.d, A.grid, sp.tn, tf);
-    if (sp.hit) sp.dt = __fdiv_rn(__fsub_rn(tf, sp.tn), static_cast<float>(A.n_samples));
+    sp.hit = ray_box(R.o, R.d, A.grid, sp.tn, sp.tf);
+    if (A.t_samples) {
+        sp.n_bins = A.n_bins;
+        bin_table(A.t_samples + ray * (int64_t)A.n_bins, A.n_bins, tab);
+        sp.dt = (sp.tf - sp.tn) / A.n_bins;
+        sp.inv_n = 1.0f / A.n_samples;
+    } else if (sp.hit) {
+        sp.dt = __fdiv_rn(__fsub_rn(sp.tf, sp.tn), static_cast<float>(A.n_samples));
+    }
     return sp;
 }
 

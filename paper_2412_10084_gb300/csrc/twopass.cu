@@ -226,8 +226,10 @@ __global__ void __launch_bounds__(kFwdThreads, 4) shade_kernel(RenderArgs A, Sha
                 float z[W];
                 tc::tmem_ld<W>(t_row + 32, z);
                 bias_relu<W>(z, f32 + M::kB2);
+                Layer3<C> l3;
+                l3.template add<W>(f32, 0, z);
                 float col[3];
-                mlp_layer3<C>(f32, z, col);
+                l3.colour(f32, col);
                 if (node >= 0) S.colours[node] = pack_colour(col);
             }
             tc::fence_before();
@@ -329,7 +331,7 @@ __global__ void __launch_bounds__(kRenderWarps * 32, 4) colour_render_kernel(
             if (!__any_sync(FULL, falls)) continue;
             float lam = 0.0f, alpha = 0.0f;
             if (falls) {
-                const float diff = log_transmittance(A.tau, s, s1, alpha);
+                const float diff = log_transmittance(A.tau, s, s1, expf(A.tau * s1), alpha);
                 if (diff < 0.0f)
                     lam = diff;
                 else
