@@ -75,8 +75,22 @@ struct BwdLayout {
     static constexpr uint32_t kTmemCols2 = kKeepBc ? 32 : 0;
     static constexpr uint32_t kBcCol = 112;
     static_assert(128 * PST * 4 <= M::kSplit * kDZ, "probe staging aliases the DZ tiles");
+    // How far the chunk loop's inner loops are unrolled.  With everything unrolled
+    // its code (107 KB in all) overran the instruction caches: at 69 % of their
+    // peak request rate the warps waited 0.56 cycles per instruction for their next
+    // one.  Rolled up (86 KB, 0.17 cycles) the object-capture adjoint takes 3 %
+    // less; wide probe rows, which wait for their gathers instead, gain nothing by
+    // it (their step 24.4 ms unrolled, 24.8 ms not), and single FP16 tiles have a
+    // third of the MMAs, so that those stay unrolled (19.9 against 20.1 ms).
+    static constexpr int kUnrollCorners = kKeepBc ? 2 : 8;
+    static constexpr int kUnrollDW3 = kKeepBc ? 4 : 8;
+    static constexpr int kUnrollDW = M::kSplit == 1 ? 8 : 1;
     static_assert(XHC <= 64, "dW accumulator fits columns 64..127");
 };
+
+// Hidden units per pass of the epilogues: a row's units are read back, biased,
+// split and stored 16 at a time by a loop (half the code and the registers).
+constexpr int kPart = 16;
 
 __device__ __forceinline__ float warp_max(float v)
 {
@@ -290,7 +304,8 @@ render_backward_kernel(RenderArgs A)
     }
     uint32_t phase = 0;
     bool bad = false, any_chunk = false, dw_started = false;
-    float acc3[3] = {0.f, 0.f, 0.f}, accb3 = 0.0f;  // dW3 column (lane % W) and db3 (lane < 3)
+    // dW3 column (lane % W) and this lane's samples' share of db3
+    float acc3[3] = {0.f, 0.f, 0.f}, accb3[3] = {0.f, 0.f, 0.f};
 
     // Per-warp work cursor: the warp's current ray and chunk.  Each CTA step
     // every warp renders one chunk (or an empty tile slice), so the barriers
@@ -307,7 +322,7 @@ render_backward_kernel(RenderArgs A)
     RaySpan sp;
     bool have = false, have_first = false;
     int ch = -1;
-    float s_first = 0.0f;
+    float s_first = 0.0f, e_first = 0.0f;
     float drgb[3] = {0.f, 0.f, 0.f}, ddepth = 0.f, dwsum = 0.f, logT_end = 0.f, s_carry = 0.f;
     const int nch = (N + 31) >> 5;
     for (;;) {
@@ -352,9 +367,10 @@ render_backward_kernel(RenderArgs A)
 
             // ---- P0: recompute geometry and features -> XH columns [0, 16) ----
             SampleGeom<C> S;
-            float t = 0.0f, lam = 0.0f, s_next = 0.0f;
+            // exp(tau s) at the sample and at the point after it
+            float t = 0.0f, lam = 0.0f, e_own = 0.0f, e_next = 0.0f;
             bool unclipped = false;
-            Cell c1;
+            Cell c1;  // the extra point's cell
             c1.base = 0;
             c1.i[0] = c1.i[1] = c1.i[2] = 0;
             c1.f[0] = c1.f[1] = c1.f[2] = 0.0f;
@@ -375,18 +391,26 @@ render_backward_kernel(RenderArgs A)
                     eval_sdf_geom<C>(A, R.o, R.d, t, S);
                 else
                     eval_sdf<C>(A, R.o, R.d, t, S);
-                s_next = __shfl_down_sync(FULL, S.s, 1);
+                e_own = expf(tau * S.s);
+                float s_next = __shfl_down_sync(FULL, S.s, 1);
+                e_next = __shfl_down_sync(FULL, e_own, 1);
                 if (extra) {
-                    if (carried)
+                    if (carried) {
                         s_next = s_first;
-                    else
-                        s_next = sdf_value(A.grid, c1);
+                        e_next = e_first;
+                    } else {
+                        SdfPoint<C::SP ? 0 : features_apart<C>() ? 1 : 4> p;
+                        p.c = c1;
+                        p.gather_cell(A.grid);
+                        s_next = p.value(A.grid);
+                        e_next = expf(tau * s_next);
+                    }
                 }
                 s_first = __shfl_sync(FULL, S.s, 0);
-                if (active) {
-                    float alpha_p;  // the adjoint takes alpha from lam
-                    const float diff =
-                        log_transmittance(tau, S.s, s_next, expf(tau * s_next), alpha_p);
+                e_first = __shfl_sync(FULL, e_own, 0);
+                if (active && s_next < S.s) {  // else the opacity is clipped to zero
+                    float alpha_p;
+                    const float diff = log_transmittance(tau, S.s, s_next, e_next, alpha_p);
                     unclipped = diff < 0.0f;
                     lam = unclipped ? diff : 0.0f;
                 }
@@ -443,21 +467,20 @@ render_backward_kernel(RenderArgs A)
             }
             const float logTk = logT_end - suf;
             const float Tk = expf(logTk);
-            const float Tk1 = expf(logTk + lam);
+            const float a_own = expf(lam);  // 1 - alpha, without its cancellation
             const float alpha = -expm1f(lam);
             bad |= !tc::mbar_wait(mbar, phase, A.wait_polls);
             phase ^= 1;
             tc::fence_after();
             uint32_t mask1 = 0;
-            {
-                float z[W];
-                tc::tmem_ld<W>(t_row + 0, z);
-                mask1 = bias_relu_mask<W>(z, f32 + M::kB1);
-                if (!have) {
+#pragma unroll 1
+            for (int u0 = 0; u0 < W; u0 += kPart) {
+                float z[kPart];
+                tc::tmem_ld<kPart>(t_row + u0, z);
+                mask1 |= bias_relu_mask<kPart>(z, f32 + M::kB1 + u0) << u0;
 #pragma unroll
-                    for (int o = 0; o < W; ++o) z[o] = 0.0f;
-                }
-                store_row<W, M::kSplit>(xhh, xhl, tid, K1, L::XHC, z);
+                for (int o = 0; o < kPart; ++o) z[o] = have ? z[o] : 0.0f;
+                store_row<kPart, M::kSplit>(xhh, xhl, tid, K1 + u0, L::XHC, z);
             }
             tc::fence_smem_to_async();
             tc::fence_before();
@@ -475,58 +498,36 @@ render_backward_kernel(RenderArgs A)
             bad |= !tc::mbar_wait(mbar, phase, A.wait_polls);
             phase ^= 1;
             tc::fence_after();
-            float h2[W];
+            // h2 also goes to the warp's rows of the DZ tiles, which are free until
+            // its dz2 row is stored: transposed (16-byte groups XOR-swizzled by row,
+            // so that both the row writes and the column reads below are free of
+            // bank conflicts), for dW3
+            float* h2s = reinterpret_cast<float*>(dzh + warp * L::kDZWarp);
             uint32_t mask2 = 0;
             float col[3];
             {
-                tc::tmem_ld<W>(t_row + 32, h2);
-                mask2 = bias_relu_mask<W>(h2, f32 + M::kB2);
                 Layer3<C> l3;
-                l3.template add<W>(f32, 0, h2);
+#pragma unroll 1
+                for (int u0 = 0; u0 < W; u0 += kPart) {
+                    float h2[kPart];
+                    tc::tmem_ld<kPart>(t_row + 32 + u0, h2);
+                    mask2 |= bias_relu_mask<kPart>(h2, f32 + M::kB2 + u0) << u0;
+                    l3.template add<kPart>(f32, u0, h2);
+#pragma unroll
+                    for (int v = 0; v < kPart / 4; ++v)
+                        *reinterpret_cast<float4*>(
+                            h2s + lane * W + 4 * ((u0 / 4 + v) ^ (lane & (W / 4 - 1)))) =
+                            make_float4(h2[4 * v], h2[4 * v + 1], h2[4 * v + 2], h2[4 * v + 3]);
+                }
                 l3.colour(f32, col);
             }
-            const float w = active ? Tk * alpha : 0.0f;
-            const float G = active ? drgb[0] * col[0] + drgb[1] * col[1] + drgb[2] * col[2] +
-                                         ddepth * t + dwsum
-                                   : 0.0f;
-            const float a_own = active ? expf(lam) : 1.0f;
-            const float b_own = active ? alpha * G : 0.0f;
-            float Am = __shfl_down_sync(FULL, a_own, 1);
-            float Bm = __shfl_down_sync(FULL, b_own, 1);
-            if (lane == 31) {
-                Am = 1.0f;
-                Bm = 0.0f;
-            }
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const float a2 = __shfl_down_sync(FULL, Am, off);
-                const float b2 = __shfl_down_sync(FULL, Bm, off);
-                if (lane + off < 32) {
-                    Bm = fmaf(Am, b2, Bm);
-                    Am = Am * a2;
-                }
-            }
-            const float Shat = fmaf(Am, s_carry, Bm);
-            const float next_carry = __shfl_sync(FULL, fmaf(a_own, Shat, b_own), 0);
-            const float dlam = unclipped ? -Tk1 * (G - Shat) : 0.0f;
-            float dlam_prev = __shfl_up_sync(FULL, dlam, 1);
-            if (lane == 0) dlam_prev = 0.0f;
-            const float ds_own = active ? (dlam_prev - dlam) * dlog_phi(tau, expf(tau * S.s)) : 0.0f;
-
+            const float w = Tk * alpha;
             float dz3[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) dz3[c] = w * drgb[c] * col[c] * (1.0f - col[c]);
-            // dW3 and db3 on the CUDA cores.  The warp's rows of the DZ tiles
-            // are free until its dz2 row is stored below: h2 goes there
-            // transposed (16-byte groups XOR-swizzled by row, so that both the
-            // row writes and the column reads are free of bank conflicts) and
-            // lane l sums column l of dz3 (x) h2 over the warp's 32 samples.
+            // dW3 and db3 on the CUDA cores: lane l sums column l of dz3 (x) h2 over
+            // the warp's 32 samples
             {
-                float* h2s = reinterpret_cast<float*>(dzh + warp * L::kDZWarp);
-#pragma unroll
-                for (int v = 0; v < W / 4; ++v)
-                    *reinterpret_cast<float4*>(h2s + lane * W + 4 * (v ^ (lane & (W / 4 - 1)))) =
-                        make_float4(h2[4 * v], h2[4 * v + 1], h2[4 * v + 2], h2[4 * v + 3]);
                 float* d3s = nullptr;
                 if constexpr (M::kSplit == 2) {
                     d3s = reinterpret_cast<float*>(dzl + warp * L::kDZWarp);
@@ -535,7 +536,7 @@ render_backward_kernel(RenderArgs A)
                 }
                 __syncwarp();
                 const int col_l = lane & (W - 1);
-#pragma unroll 8
+#pragma unroll (L::kUnrollDW3)
                 for (int r = 0; r < 32; ++r) {
                     const float h = h2s[r * W + 4 * ((col_l >> 2) ^ (r & (W / 4 - 1))) + (col_l & 3)];
                     float e0, e1, e2;
@@ -556,27 +557,27 @@ render_backward_kernel(RenderArgs A)
                 __syncwarp();
             }
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                float sb = dz3[c];
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) sb += __shfl_xor_sync(FULL, sb, off);
-                if (lane == c) accb3 += sb;
-            }
+            for (int c = 0; c < 3; ++c) accb3[c] += dz3[c];
             {
                 // dh2 = W3^T dz3 over pairs of hidden units (W3 row-major)
-                float dz2[W];
                 const float2 e0 = make_float2(dz3[0], dz3[0]), e1 = make_float2(dz3[1], dz3[1]);
                 const float2 e2 = make_float2(dz3[2], dz3[2]), sc2 = make_float2(s2, s2);
+#pragma unroll 1
+                for (int u0 = 0; u0 < W; u0 += kPart) {
+                    float dz2[kPart];
+                    const float* w3 = f32 + M::kW3 + u0;
+                    const uint32_t m = mask2 >> u0;
 #pragma unroll
-                for (int i = 0; i < W; i += 2) {
-                    float2 dh2 = mul2(*reinterpret_cast<const float2*>(f32 + M::kW3 + i), e0);
-                    dh2 = fma2(*reinterpret_cast<const float2*>(f32 + M::kW3 + W + i), e1, dh2);
-                    dh2 = fma2(*reinterpret_cast<const float2*>(f32 + M::kW3 + 2 * W + i), e2, dh2);
-                    dh2 = mul2(dh2, sc2);
-                    dz2[i] = ((mask2 >> i) & 1u) ? dh2.x : 0.0f;
-                    dz2[i + 1] = ((mask2 >> (i + 1)) & 1u) ? dh2.y : 0.0f;
+                    for (int i = 0; i < kPart; i += 2) {
+                        float2 dh2 = mul2(*reinterpret_cast<const float2*>(w3 + i), e0);
+                        dh2 = fma2(*reinterpret_cast<const float2*>(w3 + W + i), e1, dh2);
+                        dh2 = fma2(*reinterpret_cast<const float2*>(w3 + 2 * W + i), e2, dh2);
+                        dh2 = mul2(dh2, sc2);
+                        dz2[i] = ((m >> i) & 1u) ? dh2.x : 0.0f;
+                        dz2[i + 1] = ((m >> (i + 1)) & 1u) ? dh2.y : 0.0f;
+                    }
+                    store_row<kPart, M::kSplit>(dzh, dzl, tid, W + u0, L::DZC, dz2);
                 }
-                store_row<W, M::kSplit>(dzh, dzl, tid, W, L::DZC, dz2);
             }
             tc::fence_smem_to_async();
             tc::fence_before();
@@ -593,21 +594,53 @@ render_backward_kernel(RenderArgs A)
                          L::kSboDZ, (W / 8) * 128, 128, idesc, s > 0);
                 tc::commit(mbar);
             }
+            // compositing adjoint (Eq. 10), while the tensor cores work: suffix term
+            // S_k from a warp scan of the affine recurrence
+            const float G = active ? drgb[0] * col[0] + drgb[1] * col[1] + drgb[2] * col[2] +
+                                         ddepth * t + dwsum
+                                   : 0.0f;
+            const float b_own = active ? alpha * G : 0.0f;
+            float Am = __shfl_down_sync(FULL, a_own, 1);
+            float Bm = __shfl_down_sync(FULL, b_own, 1);
+            if (lane == 31) {
+                Am = 1.0f;
+                Bm = 0.0f;
+            }
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const float a2 = __shfl_down_sync(FULL, Am, off);
+                const float b2 = __shfl_down_sync(FULL, Bm, off);
+                if (lane + off < 32) {
+                    Bm = fmaf(Am, b2, Bm);
+                    Am = Am * a2;
+                }
+            }
+            const float Shat = fmaf(Am, s_carry, Bm);
+            const float next_carry = __shfl_sync(FULL, fmaf(a_own, Shat, b_own), 0);
+            const float dlam = unclipped ? -(Tk * a_own) * (G - Shat) : 0.0f;
+            float dlam_prev = __shfl_up_sync(FULL, dlam, 1);
+            if (lane == 0) dlam_prev = 0.0f;
+            const float ds_own = active ? (dlam_prev - dlam) * dlog_phi(tau, e_own) : 0.0f;
+
             bad |= !tc::mbar_wait(mbar, phase, A.wait_polls);
             phase ^= 1;
             tc::fence_after();
             {
-                float dh1[W];
-                tc::tmem_ld<W>(t_row + 0, dh1);
                 const float r12 = s1 * inv_s2;  // dh1 arrives scaled by s2; dz1 is stored scaled by s1
                 const float2 r2 = make_float2(r12, r12);
+#pragma unroll 1
+                for (int u0 = 0; u0 < W; u0 += kPart) {
+                    float dh1[kPart];
+                    tc::tmem_ld<kPart>(t_row + u0, dh1);
+                    const uint32_t m = mask1 >> u0;
 #pragma unroll
-                for (int i = 0; i < W; i += 2) {
-                    const float2 v = mul2(make_float2(dh1[i], dh1[i + 1]), r2);
-                    dh1[i] = ((mask1 >> i) & 1u) ? v.x : 0.0f;
-                    dh1[i + 1] = ((mask1 >> (i + 1)) & 1u) ? v.y : 0.0f;
+                    for (int i = 0; i < kPart; i += 2) {
+                        const float2 v = mul2(make_float2(dh1[i], dh1[i + 1]), r2);
+                        dh1[i] = ((m >> i) & 1u) ? v.x : 0.0f;
+                        dh1[i + 1] = ((m >> (i + 1)) & 1u) ? v.y : 0.0f;
+                    }
+                    store_row<kPart, M::kSplit>(dzh, dzl, tid, u0, L::DZC, dh1);
                 }
-                store_row<W, M::kSplit>(dzh, dzl, tid, 0, L::DZC, dh1);
             }
             tc::fence_smem_to_async();
             tc::fence_before();
@@ -622,7 +655,7 @@ render_backward_kernel(RenderArgs A)
                     mma_k<M::kSplit>(tmem + 32, dzh + s * 256, dzl + s * 256, w1h + s * 512, w1l + s * 512,
                          128, L::kSboDZ, 256, 128, idx, s > 0);
                 const uint32_t idw = tc::idesc_f16(64, L::XHC, 1, 1);
-#pragma unroll
+#pragma unroll (L::kUnrollDW)
                 for (int s = 0; s < 8; ++s)
                     mma_k<M::kSplit>(tmem + 64, dzh + s * 2 * L::kSboDZ, dzl + s * 2 * L::kSboDZ,
                          xhh + s * 2 * L::kSboXH, xhl + s * 2 * L::kSboXH, L::kSboDZ, 128,
@@ -630,6 +663,9 @@ render_backward_kernel(RenderArgs A)
                 dw_started = true;
                 tc::commit(mbar);
             }
+            // the blended probe coefficients come back while the tensor cores work
+            float Bc[L::kKeepBc ? L::kBc : 1];
+            if constexpr (L::kKeepBc) bc_load<L>(t_row, t_row2, Bc);  // warp-collective
             bad |= !tc::mbar_wait(mbar, phase, A.wait_polls);
             phase ^= 1;
             tc::fence_after();
@@ -654,8 +690,6 @@ render_backward_kernel(RenderArgs A)
             float* pst = reinterpret_cast<float*>(dzh) + warp * 32 * L::PST;
             if (have) {
                 float gxs = 0.0f, gys = 0.0f, gzs = 0.0f;
-                float Bc[L::kKeepBc ? L::kBc : 1];
-                if constexpr (L::kKeepBc) bc_load<L>(t_row, t_row2, Bc);  // warp-collective
                 if (unclipped) {
                     float wq[8];
                     corner_weights(S.pcell.f, wq);
@@ -729,7 +763,7 @@ render_backward_kernel(RenderArgs A)
                 }
                 if (unclipped) {
                     const float fx = S.cell.f[0], fy = S.cell.f[1], fz = S.cell.f[2];
-#pragma unroll
+#pragma unroll (L::kUnrollCorners)
                     for (int q = 0; q < 8; ++q) {
                         const int cx = q & 1, cy = (q >> 1) & 1, cz = (q >> 2) & 1;
                         const float wx = cx ? fx : 1.0f - fx, sgx = cx ? 1.0f : -1.0f;
@@ -776,27 +810,23 @@ render_backward_kernel(RenderArgs A)
                         }
                     }
                 } else if (active && ds_own != 0.0f) {
-                    float w8[8];
-                    corner_weights(S.cell.f, w8);
-#pragma unroll
+#pragma unroll 1
                     for (int q = 0; q < 8; ++q) {
                         const int64_t node = grad_record<C>(A.grid, S.cell, q);
                         if (C::SP && node < 0) continue;
                         red_add(A.grad_grid + (C::TP ? node : A.grid.rec_off + 4 * node),
-                                ds_own * w8[q]);
+                                ds_own * corner_weight(S.cell.f, q));
                     }
                 }
                 if (extra) {
-                    const float ds1 = dlam * dlog_phi(tau, expf(tau * s_next));
+                    const float ds1 = dlam * dlog_phi(tau, e_next);
                     if (ds1 != 0.0f) {
-                        float w1[8];
-                        corner_weights(c1.f, w1);
-#pragma unroll
+#pragma unroll 1
                         for (int q = 0; q < 8; ++q) {
                             const int64_t node = grad_record<C>(A.grid, c1, q);
                             if (C::SP && node < 0) continue;
                             red_add(A.grad_grid + (C::TP ? node : A.grid.rec_off + 4 * node),
-                                    ds1 * w1[q]);
+                                    ds1 * corner_weight(c1.f, q));
                         }
                     }
                 }
@@ -852,11 +882,17 @@ done:
                 gacc[C::gB2 + (r - W)] += v[NIN] * inv_s2;
             }
         }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            float sb = accb3[c];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) sb += __shfl_xor_sync(FULL, sb, off);
+            if (lane == 0) atomicAdd(gacc + C::gB3 + c, sb);
+        }
         if (lane < W) {  // lane l holds column l (see P2)
 #pragma unroll
             for (int c = 0; c < 3; ++c) atomicAdd(gacc + C::gW3 + c * W + lane, acc3[c]);
         }
-        if (lane < 3) atomicAdd(gacc + C::gB3 + lane, accb3);
     }
     tc::fence_before();
     __syncthreads();
