@@ -100,13 +100,16 @@ __device__ __forceinline__ float warp_max(float v)
 }
 
 // Probe-coefficient gradient (Eqs. 6-7): dL/db_ijc = sum_k w_i(k) Y_j(k) dF_a,c(k).
-// Samples of a chunk that share a probe cell are consecutive; lane (corner i,
-// channel c) sums each run over the rows in `live` and issues one reduction
-// per coefficient at the run's last sample (the bits of `ends`).  The next
-// row's operands are loaded while the current row is summed.
+// The warp's n live samples are staged in consecutive rows; those that share a
+// probe cell follow one another.  Lane (corner i, channel c) sums each run and
+// issues one reduction per coefficient at the run's last row (the bits of
+// `ends`).  The operands of kBatch rows are read before the first is summed: the
+// loop is bound by its shared-memory latency, not by the reductions (one row
+// ahead, at rows found bit by bit, it took 1.0 of the object-capture adjoint's
+// 5.9 ms; without its reductions it took as long).
 template <class C, int PST>
-__device__ __forceinline__ void scatter_probe_grad(const RenderArgs& A, const float* pst,
-                                                   uint32_t live, uint32_t ends, int lane)
+__device__ __forceinline__ void scatter_probe_grad(const RenderArgs& A, const float* pst, int n,
+                                                   uint32_t ends, int lane)
 {
     constexpr int L2 = C::L2, NA = C::NA;
     constexpr int CPL = (8 * NA) / 32;
@@ -114,69 +117,65 @@ __device__ __forceinline__ void scatter_probe_grad(const RenderArgs& A, const fl
     static_assert(PST % 4 == 0, "rows of whole 16-byte vectors");
     constexpr int L2V = (L2 + 3) / 4;  // Y_j starts at float 8: 16-byte aligned
     static_assert(8 + 4 * L2V <= PST, "vector reads stay inside the row");
-    if (!live) return;
+    constexpr int kBatch = L2V * CPL <= 3 ? 4 : 2;
+    static_assert(32 % kBatch == 0, "batches stay inside the 32 rows");
     const int Px = A.probes.P[0], Pxy = A.probes.P[0] * A.probes.P[1];
-    int q[CPL], ch[CPL], qoff[CPL];
+    int q[CPL], ch[CPL], off[CPL];
     float acc[CPL][L2];
 #pragma unroll
     for (int m = 0; m < CPL; ++m) {
         const int combo = lane + 32 * m;
         q[m] = combo / NA;
         ch[m] = combo % NA;
-        qoff[m] = (q[m] & 1) + ((q[m] >> 1) & 1) * Px + ((q[m] >> 2) & 1) * Pxy;
+        off[m] = ((q[m] & 1) + ((q[m] >> 1) & 1) * Px + ((q[m] >> 2) & 1) * Pxy) * (L2 * NA) + ch[m];
 #pragma unroll
         for (int j = 0; j < L2; ++j) acc[m][j] = 0.f;
     }
-    // row s: w_i at [0, 8), Y_j at 8, dF_a at 8 + L2, the probe cell at 8 + L2 + NA
-    auto load = [&](int s, float4 (&y)[L2V], float (&coef)[CPL]) {
-        const float* row = pst + s * PST;
+    // row: w_i at [0, 8), Y_j at 8, dF_a at 8 + L2, the probe cell at 8 + L2 + NA
+#pragma unroll 1
+    for (int r0 = 0; r0 < n; r0 += kBatch) {
+        const float* row = pst + r0 * PST;
+        float4 y[kBatch][L2V];
+        float coef[kBatch][CPL];
 #pragma unroll
-        for (int v = 0; v < L2V; ++v) y[v] = *reinterpret_cast<const float4*>(row + 8 + 4 * v);
+        for (int i = 0; i < kBatch; ++i) {  // rows past the last are read, not used
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) coef[m] = row[q[m]] * row[8 + L2 + ch[m]];
-    };
-    int s = __ffs(live) - 1;
-    uint32_t rem = live & (live - 1);
-    float4 y[L2V];
-    float coef[CPL];
-    load(s, y, coef);
-    for (;;) {
-        const int sn = rem ? __ffs(rem) - 1 : s;
-        float4 yn[L2V];
-        float coefn[CPL];
-        load(sn, yn, coefn);
-        const float* Y = reinterpret_cast<const float*>(y);
+            for (int v = 0; v < L2V; ++v)
+                y[i][v] = *reinterpret_cast<const float4*>(row + i * PST + 8 + 4 * v);
 #pragma unroll
-        for (int m = 0; m < CPL; ++m) {
-            const float2 c2 = make_float2(coef[m], coef[m]);
-#pragma unroll
-            for (int j = 0; j + 1 < L2; j += 2) {
-                const float2 r = fma2(c2, make_float2(Y[j], Y[j + 1]),
-                                      make_float2(acc[m][j], acc[m][j + 1]));
-                acc[m][j] = r.x;
-                acc[m][j + 1] = r.y;
-            }
-            if constexpr (L2 % 2) acc[m][L2 - 1] = fmaf(coef[m], Y[L2 - 1], acc[m][L2 - 1]);
+            for (int m = 0; m < CPL; ++m)
+                coef[i][m] = row[i * PST + q[m]] * row[i * PST + 8 + L2 + ch[m]];
         }
-        if ((ends >> s) & 1u) {
-            const int cell = __float_as_int(pst[s * PST + 8 + L2 + NA]);
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+            if (r0 + i >= n) break;
+            const float* Y = reinterpret_cast<const float*>(y[i]);
 #pragma unroll
             for (int m = 0; m < CPL; ++m) {
-                float* dst = A.grad_probes + (size_t)(cell + qoff[m]) * (L2 * NA) + ch[m];
+                const float2 c2 = make_float2(coef[i][m], coef[i][m]);
 #pragma unroll
-                for (int j = 0; j < L2; ++j) {
-                    red_add(dst + j * NA, acc[m][j]);
-                    acc[m][j] = 0.f;
+                for (int j = 0; j + 1 < L2; j += 2) {
+                    const float2 r = fma2(c2, make_float2(Y[j], Y[j + 1]),
+                                          make_float2(acc[m][j], acc[m][j + 1]));
+                    acc[m][j] = r.x;
+                    acc[m][j + 1] = r.y;
+                }
+                if constexpr (L2 % 2) acc[m][L2 - 1] = fmaf(coef[i][m], Y[L2 - 1], acc[m][L2 - 1]);
+            }
+            if ((ends >> (r0 + i)) & 1u) {
+                const int64_t cell =
+                    int64_t(__float_as_int(row[i * PST + 8 + L2 + NA])) * (L2 * NA);
+#pragma unroll
+                for (int m = 0; m < CPL; ++m) {
+                    float* dst = A.grad_probes + cell + off[m];
+#pragma unroll
+                    for (int j = 0; j < L2; ++j) {
+                        red_add(dst + j * NA, acc[m][j]);
+                        acc[m][j] = 0.f;
+                    }
                 }
             }
         }
-        if (!rem) break;
-        rem &= rem - 1;
-        s = sn;
-#pragma unroll
-        for (int v = 0; v < L2V; ++v) y[v] = yn[v];
-#pragma unroll
-        for (int m = 0; m < CPL; ++m) coef[m] = coefn[m];
     }
 }
 
@@ -689,6 +688,7 @@ render_backward_kernel(RenderArgs A)
             // transmittance term (ds_own), skipped when that is zero too.
             float* pst = reinterpret_cast<float*>(dzh) + warp * 32 * L::PST;
             if (have) {
+                const uint32_t live = __ballot_sync(FULL, unclipped);
                 float gxs = 0.0f, gys = 0.0f, gzs = 0.0f;
                 if (unclipped) {
                     float wq[8];
@@ -726,7 +726,8 @@ render_backward_kernel(RenderArgs A)
                     {
                         float Y[L2];
                         sh_basis<L2>(S.r, Y);
-                        float* row = pst + lane * L::PST;
+                        // live samples in consecutive rows
+                        float* row = pst + __popc(live & ((1u << lane) - 1u)) * L::PST;
 #pragma unroll
                         for (int q = 0; q < 8; ++q) row[q] = wq[q];
 #pragma unroll
@@ -832,15 +833,15 @@ render_backward_kernel(RenderArgs A)
                 }
                 // runs of live samples in one probe cell end where the next live
                 // sample's cell differs (or no live sample follows)
-                const uint32_t live = __ballot_sync(FULL, unclipped);
                 const int my_cell = unclipped ? S.pcell.base : -1;
                 const uint32_t later = lane == 31 ? 0u : live & (0xffffffffu << (lane + 1));
                 const int nl = __ffs(later) - 1;
                 const int next_cell = __shfl_sync(FULL, my_cell, nl >= 0 ? nl : lane);
-                const uint32_t ends =
-                    __ballot_sync(FULL, unclipped && (nl < 0 || next_cell != my_cell));
+                const bool last = unclipped && (nl < 0 || next_cell != my_cell);
+                const uint32_t ends = __reduce_or_sync(
+                    FULL, last ? 1u << __popc(live & ((1u << lane) - 1u)) : 0u);
                 __syncwarp();
-                scatter_probe_grad<C, L::PST>(A, pst, live, ends, lane);
+                scatter_probe_grad<C, L::PST>(A, pst, __popc(live), ends, lane);
                 logT_end = __shfl_sync(FULL, logTk, 0);
                 s_carry = next_carry;
                 have_first = true;
