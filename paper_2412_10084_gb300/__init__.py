@@ -578,6 +578,7 @@ class RenderFunction(torch.autograd.Function):
         ctx.params = params
         ctx.check_status = check_status
         ctx.mark_non_differentiable(logT, live)
+        ctx.set_materialize_grads(False)  # an output without a cotangent costs nothing
         return rgb, depth, wsum
 
     @staticmethod

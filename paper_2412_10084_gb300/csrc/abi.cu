@@ -433,6 +433,28 @@ cudaError_t set_smem_carveout(const void* func, int threads, size_t dyn_smem, un
     return cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
 }
 
+cudaError_t prepare_kernel(const void* func, int threads, size_t dyn_smem, unsigned tmem_cols,
+                           KernelCache& cache, int* ctas_per_sm)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool keep = dev >= 0 && dev < kMaxDevices;
+    if (keep && (*ctas_per_sm = cache.ctas[dev].load(std::memory_order_acquire)) > 0)
+        return cudaSuccess;
+    e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(dyn_smem));
+    if (e == cudaSuccess) e = set_smem_carveout(func, threads, dyn_smem, tmem_cols);
+    cudaFuncAttributes fa;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, func);
+    if (e != cudaSuccess) return e;
+    const int n = resident_ctas(fa, threads, dyn_smem, tmem_cols);
+    if (n <= 0) return cudaErrorInvalidConfiguration;
+    if (keep) cache.ctas[dev].store(n, std::memory_order_release);
+    *ctas_per_sm = n;
+    return cudaSuccess;
+}
+
 cudaError_t launch_pack(const float* sdf, const float* feat, float4* packed, int64_t n_nodes,
                         cudaStream_t stream)
 {
@@ -542,8 +564,10 @@ psdf_status psdf_device_status(void* stream, int32_t* flags)
     int v = 0;
     cudaError_t e = cudaMemcpyAsync(&v, p, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && v != 0) {  // a clear word needs no clearing
+        e = cudaMemsetAsync(p, 0, sizeof(int), s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    }
     if (e != cudaSuccess) return cuda_status(e);
     *flags = v;
     return PSDF_OK;

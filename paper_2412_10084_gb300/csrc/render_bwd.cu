@@ -909,12 +909,6 @@ template <class C>
 cudaError_t launch_backward_t(const RenderArgs& A, int grid_ctas, cudaStream_t stream)
 {
     using L = BwdLayout<C>;
-    cudaError_t e = cudaFuncSetAttribute(render_backward_kernel<C>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes);
-    if (e == cudaSuccess)
-        e = set_smem_carveout(reinterpret_cast<const void*>(render_backward_kernel<C>),
-                              kBwdThreads, L::kBytes, L::kTmemCols + L::kTmemCols2);
-    if (e != cudaSuccess) return e;
     render_backward_kernel<C><<<grid_ctas, kBwdThreads, L::kBytes, stream>>>(A);
     return cudaGetLastError();
 }
@@ -934,14 +928,9 @@ template <class C>
 cudaError_t backward_occupancy_t(int* n)
 {
     using L = BwdLayout<C>;
-    cudaError_t e = cudaFuncSetAttribute(render_backward_kernel<C>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes);
-    if (e != cudaSuccess) return e;
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, render_backward_kernel<C>);
-    if (e != cudaSuccess) return e;
-    *n = resident_ctas(fa, kBwdThreads, L::kBytes, L::kTmemCols + L::kTmemCols2);
-    return *n > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
+    static KernelCache cache;
+    return prepare_kernel(reinterpret_cast<const void*>(render_backward_kernel<C>), kBwdThreads, L::kBytes,
+                          L::kTmemCols + L::kTmemCols2, cache, n);
 }
 
 cudaError_t backward_ctas_per_sm(const KernelShape& ks, int* n)

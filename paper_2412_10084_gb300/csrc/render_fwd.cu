@@ -330,12 +330,6 @@ template <class C>
 cudaError_t launch_forward_t(const RenderArgs& A, int grid_ctas, cudaStream_t stream)
 {
     using L = FwdLayout<C>;
-    cudaError_t e = cudaFuncSetAttribute(render_forward_kernel<C>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes);
-    if (e == cudaSuccess)
-        e = set_smem_carveout(reinterpret_cast<const void*>(render_forward_kernel<C>),
-                              kFwdThreads, L::kBytes, L::kTmemCols);
-    if (e != cudaSuccess) return e;
     render_forward_kernel<C><<<grid_ctas, kFwdThreads, L::kBytes, stream>>>(A);
     return cudaGetLastError();
 }
@@ -355,14 +349,9 @@ template <class C>
 cudaError_t forward_occupancy_t(int* n)
 {
     using L = FwdLayout<C>;
-    cudaError_t e = cudaFuncSetAttribute(render_forward_kernel<C>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes);
-    if (e != cudaSuccess) return e;
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, render_forward_kernel<C>);
-    if (e != cudaSuccess) return e;
-    *n = resident_ctas(fa, kFwdThreads, L::kBytes, L::kTmemCols);
-    return *n > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
+    static KernelCache cache;
+    return prepare_kernel(reinterpret_cast<const void*>(render_forward_kernel<C>), kFwdThreads, L::kBytes,
+                          L::kTmemCols, cache, n);
 }
 
 cudaError_t forward_ctas_per_sm(const KernelShape& ks, int* n)
