@@ -783,7 +783,7 @@ int dense_chunk(int64_t tiles, int Rz, int resident, int extra)
     const int64_t slots = int64_t(sms()) * resident;
     int best = Rz;
     int64_t cost = INT64_MAX;
-    for (int n = 1; n <= (Rz + 7) / 8 && n <= 65535; ++n) {
+    for (int n = 1; n <= (Rz + 3) / 4 && n <= 65535; ++n) {
         const int zc = (Rz + n - 1) / n;
         const int64_t waves = (tiles * ((Rz + zc - 1) / zc) + slots - 1) / slots;
         if (waves * (zc + extra) < cost) {
