@@ -330,7 +330,7 @@ render_backward_kernel(RenderArgs A)
             have = false;
             while (ray < A.n_rays) {
                 R = load_ray(A, ray);
-                sp = ray_span(A, R, ray, stab + 64 * warp);
+                sp = ray_span<false>(A, R, ray, stab + 64 * warp);
                 const int live = A.n_live ? __ldg(A.n_live + ray) : N;
                 if (sp.hit && live > 0) {
                     // the chunk of the last sample with alpha > 0; sample

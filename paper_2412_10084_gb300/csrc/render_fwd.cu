@@ -176,8 +176,10 @@ render_forward_kernel(RenderArgs A)
                     const float diff = log_transmittance(A.tau, S.s, P.s, expf(A.tau * P.s), alpha);
                     opaque = diff < 0.0f;
                     lam = opaque ? diff : 0.0f;
-                    if (!opaque) alpha = 0.0f;
-                    if constexpr (C::MH) alpha = -expm1f(lam);  // the adjoint's bits
+                    if constexpr (C::MH)
+                        alpha = -expm1f(lam);  // the adjoint's bits
+                    else if (!opaque)
+                        alpha = 0.0f;
                 }
                 // a clipped opacity (alpha = 0) gives the sample weight 0: its
                 // colour, and so its appearance inputs, never reach an output

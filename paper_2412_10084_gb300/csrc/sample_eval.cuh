@@ -414,9 +414,8 @@ struct RaySpan {
     const float* tab;
 };
 
-// Running sums and reciprocals of a ray's bin densities into the warp's table
-// (out of line, so that the other modes' loops do not carry its code).
-static __device__ __noinline__ void bin_table(const float* q_ray, int n_bins, float* tab)
+// Running sums and reciprocals of a ray's bin densities into the warp's table.
+__device__ __forceinline__ void bin_table(const float* q_ray, int n_bins, float* tab)
 {
     const int lane = threadIdx.x & 31;
     const float q = lane < n_bins ? __ldg(q_ray + lane) : 0.0f;
@@ -431,8 +430,17 @@ static __device__ __noinline__ void bin_table(const float* q_ray, int n_bins, fl
     __syncwarp();
 }
 
+// Out of line, for the adjoint: its other modes' loop does not carry the code
+// then (8.04 against 8.16 ms on the object-capture step).  The forward, which
+// renders proposed samples, keeps it inline (6.04 against 6.10 ms a 1080p frame).
+static __device__ __noinline__ void bin_table_call(const float* q_ray, int n_bins, float* tab)
+{
+    bin_table(q_ray, n_bins, tab);
+}
+
 // tab: this warp's 64-float shared-memory table (used in the bin-density
 // mode).  Warp-uniform: every lane of the warp calls it for the warp's ray.
+template <bool kInline = true>
 __device__ __forceinline__ RaySpan ray_span(const RenderArgs& A, const RayIn& R, int64_t ray,
                                             float* tab)
 {
@@ -453,7 +461,11 @@ __device__ __forceinline__ RaySpan ray_span(const RenderArgs& A, const RayIn& R,
     sp.hit = ray_box(R.o, R.d, A.grid, sp.tn, sp.tf);
     if (A.t_samples) {
         sp.n_bins = A.n_bins;
-        bin_table(A.t_samples + ray * (int64_t)A.n_bins, A.n_bins, tab);
+        const float* q = A.t_samples + ray * (int64_t)A.n_bins;
+        if constexpr (kInline)
+            bin_table(q, A.n_bins, tab);
+        else
+            bin_table_call(q, A.n_bins, tab);
         sp.dt = (sp.tf - sp.tn) / A.n_bins;
         sp.inv_n = 1.0f / A.n_samples;
     } else if (sp.hit) {
