@@ -11,11 +11,11 @@
 //   P0  recompute geometry and features -> input row of the XH tile;
 //   P1  layer 1 (tensor cores); warp suffix sum of the clipped log-opacities
 //       gives log T_k;
-//   P2  layer 2 (tensor cores) and layer 3; the suffix term of
-//       dL/dalpha_k = T_k (G_k - S_k) from a warp scan of the affine recurrence
-//       S_k = alpha_{k+1} G_{k+1} + (1 - alpha_{k+1}) S_{k+1}; sigmoid and layer-3
-//       adjoints on the CUDA cores -> dz2 row of the DZ tile;
-//   P3  dh1 = dz2 W2 (tensor cores, W2 read transposed) -> dz1 row;
+//   P2  layer 2 (tensor cores) and layer 3; sigmoid and layer-3 adjoints on the
+//       CUDA cores -> dz2 row of the DZ tile;
+//   P3  dh1 = dz2 W2 (tensor cores, W2 read transposed) -> dz1 row; meanwhile the
+//       suffix term of dL/dalpha_k = T_k (G_k - S_k) from a warp scan of the affine
+//       recurrence S_k = alpha_{k+1} G_{k+1} + (1 - alpha_{k+1}) S_{k+1};
 //   P4  dx = dz1 W1 (tensor cores) and the weight gradient
 //       [dz1 | dz2]^T [x, 1 | h1] as an M = 64 MMA over the transposed tiles,
 //       accumulated in tensor memory for the whole kernel;

@@ -398,20 +398,6 @@ __device__ __forceinline__ int gather_corners_sparse(const GridView& g, const Ce
     return stored;
 }
 
-// The 8 corner SDF values of a cell of a dense grid (FP32 node records, or
-// the SDF array of the BF16-feature and tri-plane layouts), loaded but not yet
-// combined, so that a caller can have them in flight with other loads.
-__device__ __forceinline__ void sdf_corners_load(const GridView& g, const Cell& c, float v[8])
-{
-    const int sx = 1, sy = g.R[0], sz = g.R[0] * g.R[1];
-    const bool split = g.sdf != nullptr;  // BF16-feature layout: SDF in its own array
-    const float* p = split ? g.sdf + c.base : reinterpret_cast<const float*>(g.nodes + c.base);
-    const int st = split ? 1 : 4;
-    const int off[8] = {0, sx, sy, sx + sy, sz, sz + sx, sz + sy, sz + sy + sx};
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = __ldg(p + st * off[q]);
-}
-
 // Trilinear SDF value from the corner values: the same weights and summation
 // order as sdf_full, so both give the same bits for the same point.
 __device__ __forceinline__ float sdf_corners_combine(const Cell& c, const float v[8])
@@ -424,30 +410,9 @@ __device__ __forceinline__ float sdf_corners_combine(const Cell& c, const float 
     return s;
 }
 
-// SDF value only (the point after a chunk's last sample).
-__device__ __forceinline__ float sdf_value(const GridView& g, const Cell& c)
-{
-    if (g.table) {
-        int64_t rec[8];
-        if (brick_corners(g, c.i, rec) == 0) return g.empty_sdf;
-        float w[8];
-        corner_weights(c.f, w);
-        float s = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-            s = fmaf(w[q], rec[q] >= 0 ? __ldg(reinterpret_cast<const float*>(g.nodes + rec[q]))
-                                       : g.empty_sdf,
-                     s);
-        return s;
-    }
-    float v[8];
-    sdf_corners_load(g, c, v);
-    return sdf_corners_combine(c, v);
-}
-
 // SDF of a point in two halves, the gather and the interpolation, so that a march
 // can have the next points' gathers in flight while it works on the current ones.
-// The value has the bits of sdf_value.  STRIDE: floats between the SDF values of
+// The value has the bits of sdf_full's.  STRIDE: floats between the SDF values of
 // x-neighbours (4 in FP32 node records, 1 in an array of their own); 0: sparse.
 template <int STRIDE>
 struct SdfPoint {
