@@ -36,12 +36,9 @@ struct MlpTC {
 
 // Cooperative load of the packed FP32 parameters into the split weight tiles
 // (hi at w, lo at w + kW1 / + kW2) and the FP32 block.
-// BIAS1: b1 goes into the columns NIN (its FP16 part) and NIN + 1 (the rest) of
-// W1's hi tile, for input rows that hold 1 in both.
-template <class C, bool BIAS1 = false>
+template <class C>
 __device__ __forceinline__ void load_mlp_tc(const float* __restrict__ g, uint8_t* wt, float* f32)
 {
-    static_assert(C::NIN + 2 <= MlpTC<C>::K1, "two bias columns");
     using M = MlpTC<C>;
     constexpr int W = C::W;
     uint8_t* w1h = M::w1h(wt);
@@ -53,11 +50,6 @@ __device__ __forceinline__ void load_mlp_tc(const float* __restrict__ g, uint8_t
         const float v = j < C::NIN ? g[C::gW1 + o * C::NIN + j] : 0.0f;
         __half h, l;
         tc::split2(v, h, l);
-        if (BIAS1 && (j == C::NIN || j == C::NIN + 1)) {
-            tc::split2(g[C::gB1 + o], h, l);
-            if (j == C::NIN + 1) h = l;
-            l = __float2half_rn(0.0f);
-        }
         const uint32_t off = tc::tile_off(o, j, M::K1);
         *reinterpret_cast<__half*>(w1h + off) = h;
         if constexpr (M::kSplit == 2) *reinterpret_cast<__half*>(w1l + off) = l;
@@ -157,14 +149,6 @@ __device__ __forceinline__ void bias_relu(float* z, const float* b)
         z[o] = fmaxf(h.x, 0.0f);
         z[o + 1] = fmaxf(h.y, 0.0f);
     }
-}
-
-// z = max(z, 0): the bias is already in the accumulator.
-template <int NV>
-__device__ __forceinline__ void relu(float* z)
-{
-#pragma unroll
-    for (int o = 0; o < NV; ++o) z[o] = fmaxf(z[o], 0.0f);
 }
 
 // bias_relu that also returns the mask of the units with z + b > 0.

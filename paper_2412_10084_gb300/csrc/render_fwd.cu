@@ -21,9 +21,11 @@
 //
 // Bound: the L1 data pipe (76 % of its active cycles: 72 16-byte probe loads a
 // sample, and the CUDA-core layers' parameters from shared memory) and gather
-// latency.  Measured on a 1080p view, 256 samples: 9.5 ms against 10.0 ms with
-// every chunk's opacities evaluated, alpha from an expm1 of its own, two shuffles
-// a value for the one-sample shift, and the first bias added on the CUDA cores.
+// latency.  Measured on a 1080p view, 256 samples: 9.6 ms against 9.9 ms with
+// every chunk's opacities evaluated, alpha from an expm1 of its own and two
+// shuffles a value for the one-sample shift.  Layer 1's bias is an FP32 addition
+// on the CUDA cores: as two FP16 columns of the MMA it took 0.15 ms less, but
+// had 22 bits and FP16's range.
 #include "internal.h"
 #include "mlp_tc.cuh"
 
@@ -47,10 +49,6 @@ struct FwdLayout {
     // 32 columns per warp: layer 1's accumulator, then layer 2's over it
     static constexpr uint32_t kTmemCols = 128;
     static_assert(C::W <= 32, "a warp's accumulator fits its 32 columns");
-    // Layer 1's bias comes with the MMA (two input columns of ones) instead of 32
-    // shared-memory reads and additions a sample.  Not with single FP16 tiles: a
-    // last-bit change of the colours there moves FP16 roundings of the adjoint.
-    static constexpr bool kBias1 = !C::MH;
 };
 
 template <class C>
@@ -73,7 +71,7 @@ render_forward_kernel(RenderArgs A)
     int* ray_counter = reinterpret_cast<int*>(smem + L::oBar + 36);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    load_mlp_tc<C, L::kBias1>(A.mlp, wt, f32);
+    load_mlp_tc<C>(A.mlp, wt, f32);
     if (warp == 0) tc::tmem_alloc(tslot, L::kTmemCols);
     if (tid < 4) tc::mbar_init(mbars + tid, 1);
     if (tid == 0) *ray_counter = 0;
@@ -193,9 +191,7 @@ render_forward_kernel(RenderArgs A)
                 if (__any_sync(FULL, lam < 0.0f)) {
                     float xin[M::K1];
 #pragma unroll
-                    for (int i = 0; i < M::K1; ++i)
-                        xin[i] = i < C::NIN ? S.x[i]
-                                 : (L::kBias1 && i < C::NIN + 2 ? 1.0f : 0.0f);
+                    for (int i = 0; i < M::K1; ++i) xin[i] = i < C::NIN ? S.x[i] : 0.0f;
                     store_row<M::K1, M::kSplit>(xh, xl, tid, 0, M::K1, xin);
                 }
             }
@@ -243,10 +239,7 @@ render_forward_kernel(RenderArgs A)
             {
                 float z[W];
                 tc::tmem_ld<W>(t_row, z);
-                if constexpr (L::kBias1)
-                    relu<W>(z);
-                else
-                    bias_relu<W>(z, f32 + M::kB1);
+                bias_relu<W>(z, f32 + M::kB1);
                 store_row<W, M::kSplit>(hh, hl, tid, 0, W, z);
             }
             // the layer-1 reads are complete (tcgen05.wait::ld) before the
