@@ -928,9 +928,8 @@ template <class C>
 cudaError_t backward_occupancy_t(int* n)
 {
     using L = BwdLayout<C>;
-    static KernelCache cache;
     return prepare_kernel(reinterpret_cast<const void*>(render_backward_kernel<C>), kBwdThreads, L::kBytes,
-                          L::kTmemCols + L::kTmemCols2, cache, n);
+                          L::kTmemCols + L::kTmemCols2, n);
 }
 
 cudaError_t backward_ctas_per_sm(const KernelShape& ks, int* n)
