@@ -542,8 +542,6 @@ __global__ void __launch_bounds__(T::kThreads, SPARSE ? 2 : 1) sdf_reg_kernel(Sd
             constexpr bool kInner = decltype(inner)::value;
             const int zo = z - 3;
             const int e_out = e[(u + 3) % 6];
-            copy_wait<kAhead - 1>();
-            __syncthreads();  // plane z has landed; N of plane z - 2 and G of z - 3 are written
             if (kInner || z + kAhead < z1 + H) {
                 walk(z + kAhead, (u + kAhead) % 6);
                 fetch(inner, z + kAhead, (u + kAhead) % 6);
@@ -650,6 +648,10 @@ __global__ void __launch_bounds__(T::kThreads, SPARSE ? 2 : 1) sdf_reg_kernel(Sd
             for (int u = 0; u < 6; ++u) {
                 const int z = zs + u;
                 if (z >= z1 + H) break;
+                copy_wait<kAhead - 1>();
+                // plane z has landed; N of plane z - 2 and G of z - 3 are written.  The
+                // one barrier of a step, ahead of the branch, which differs by warp.
+                __syncthreads();
                 if (full && z >= lo && z < hi)
                     step(Yes(), u, z);
                 else
