@@ -25,7 +25,7 @@ struct psdf_mlp {
     const void* params;
 };
 
-// Device status word (per context, static storage): kernels OR error bits into
+// Device status word (per device, static storage): kernels OR error bits into
 // it; psdf_device_status reads and clears it.
 __device__ int g_device_status;
 
@@ -35,12 +35,18 @@ thread_local int32_t g_last_cuda_error = 0;
 // Polls of each tensor-core completion wait in the kernels this thread launches.
 thread_local uint32_t g_wait_polls = psdf::tc::kWaitPolls;
 
-// Address of g_device_status in the current context.
+// Address of g_device_status on the current device (looked up once per device).
 int* device_status_ptr()
 {
-    void* p = nullptr;
-    return cudaGetSymbolAddress(&p, g_device_status) == cudaSuccess ? static_cast<int*>(p)
-                                                                    : nullptr;
+    static int* ptrs[64] = {nullptr};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    if (!ptrs[dev]) {
+        void* p = nullptr;
+        if (cudaGetSymbolAddress(&p, g_device_status) != cudaSuccess) return nullptr;
+        ptrs[dev] = static_cast<int*>(p);
+    }
+    return ptrs[dev];
 }
 
 psdf_status cuda_status(cudaError_t e)
@@ -428,21 +434,23 @@ cudaError_t set_smem_carveout(const void* func, int threads, size_t dyn_smem, un
 }
 
 cudaError_t prepare_kernel(const void* func, int threads, size_t dyn_smem, unsigned tmem_cols,
-                           int* ctas_per_sm)
+                           KernelCache& cache, int* ctas_per_sm)
 {
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, func);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (fa.maxDynamicSharedSizeBytes != static_cast<int>(dyn_smem)) {
-        // the size last: it marks the kernel as prepared
-        e = set_smem_carveout(func, threads, dyn_smem, tmem_cols);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(dyn_smem));
-        if (e != cudaSuccess) return e;
-    }
+    const bool keep = dev >= 0 && dev < kMaxDevices;
+    if (keep && (*ctas_per_sm = cache.ctas[dev].load(std::memory_order_acquire)) > 0)
+        return cudaSuccess;
+    e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(dyn_smem));
+    if (e == cudaSuccess) e = set_smem_carveout(func, threads, dyn_smem, tmem_cols);
+    cudaFuncAttributes fa;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, func);
+    if (e != cudaSuccess) return e;
     const int n = resident_ctas(fa, threads, dyn_smem, tmem_cols);
     if (n <= 0) return cudaErrorInvalidConfiguration;
+    if (keep) cache.ctas[dev].store(n, std::memory_order_release);
     *ctas_per_sm = n;
     return cudaSuccess;
 }

@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "render_common.cuh"
 
 namespace psdf {
@@ -54,13 +56,18 @@ int resident_ctas(const cudaFuncAttributes& fa, int threads, size_t dyn_smem, un
 // so that the rest of the SM's on-chip memory serves its gathers as L1.
 cudaError_t set_smem_carveout(const void* func, int threads, size_t dyn_smem, unsigned tmem_cols);
 
-// Prepares a kernel for launches in the current context (dynamic shared memory,
-// carveout) and returns its resident CTAs per SM.  The attributes belong to the
-// context (a reset or a second context starts without them), so they are read on
-// every call and set only where they are missing (a forward call of 64 rays takes the
-// host 3.5 us, 4.8 us with them set every time).
+// Prepares a kernel for launches on the current device (dynamic shared memory,
+// carveout) and returns its resident CTAs per SM.  Both are properties of the
+// kernel and the device alone, so they are set and computed once per device and
+// kept in `cache` (zero-initialised, one per kernel): the attribute calls took
+// longer than the launch.  Threads that meet here for the first time do the same
+// work twice.
+constexpr int kMaxDevices = 64;
+struct KernelCache {
+    std::atomic<int> ctas[kMaxDevices];
+};
 cudaError_t prepare_kernel(const void* func, int threads, size_t dyn_smem, unsigned tmem_cols,
-                           int* ctas_per_sm);
+                           KernelCache& cache, int* ctas_per_sm);
 
 // Resident CTAs per SM of a render kernel (occupancy, capped by tensor-memory
 // columns); called before its launch_ function, which sets no attribute.

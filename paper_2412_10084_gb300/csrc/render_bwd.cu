@@ -928,8 +928,9 @@ template <class C>
 cudaError_t backward_occupancy_t(int* n)
 {
     using L = BwdLayout<C>;
+    static KernelCache cache;
     return prepare_kernel(reinterpret_cast<const void*>(render_backward_kernel<C>), kBwdThreads, L::kBytes,
-                          L::kTmemCols + L::kTmemCols2, n);
+                          L::kTmemCols + L::kTmemCols2, cache, n);
 }
 
 cudaError_t backward_ctas_per_sm(const KernelShape& ks, int* n)

@@ -344,8 +344,9 @@ template <class C>
 cudaError_t forward_occupancy_t(int* n)
 {
     using L = FwdLayout<C>;
+    static KernelCache cache;
     return prepare_kernel(reinterpret_cast<const void*>(render_forward_kernel<C>), kFwdThreads, L::kBytes,
-                          L::kTmemCols, n);
+                          L::kTmemCols, cache, n);
 }
 
 cudaError_t forward_ctas_per_sm(const KernelShape& ks, int* n)
