@@ -25,7 +25,7 @@ struct psdf_mlp {
     const void* params;
 };
 
-// Device status word (per device, static storage): kernels OR error bits into
+// Device status word (per context, static storage): kernels OR error bits into
 // it; psdf_device_status reads and clears it.
 __device__ int g_device_status;
 
@@ -35,18 +35,13 @@ thread_local int32_t g_last_cuda_error = 0;
 // Polls of each tensor-core completion wait in the kernels this thread launches.
 thread_local uint32_t g_wait_polls = psdf::tc::kWaitPolls;
 
-// Address of g_device_status on the current device (looked up once per device).
+// Address of g_device_status in the current context.  It is asked for on every
+// call: another context on the device has it elsewhere.
 int* device_status_ptr()
 {
-    static int* ptrs[64] = {nullptr};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    if (!ptrs[dev]) {
-        void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_device_status) != cudaSuccess) return nullptr;
-        ptrs[dev] = static_cast<int*>(p);
-    }
-    return ptrs[dev];
+    void* p = nullptr;
+    return cudaGetSymbolAddress(&p, g_device_status) == cudaSuccess ? static_cast<int*>(p)
+                                                                    : nullptr;
 }
 
 psdf_status cuda_status(cudaError_t e)

@@ -60,8 +60,9 @@ cudaError_t set_smem_carveout(const void* func, int threads, size_t dyn_smem, un
 // carveout) and returns its resident CTAs per SM.  Both are properties of the
 // kernel and the device alone, so they are set and computed once per device and
 // kept in `cache` (zero-initialised, one per kernel): the attribute calls took
-// longer than the launch.  Threads that meet here for the first time do the same
-// work twice.
+// longer than the launch.  The runtime carries the attributes over to the
+// device's other contexts and past a reset of the device.  Threads that meet here
+// for the first time do the same work twice.
 constexpr int kMaxDevices = 64;
 struct KernelCache {
     std::atomic<int> ctas[kMaxDevices];
