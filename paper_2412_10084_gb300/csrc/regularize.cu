@@ -369,10 +369,11 @@ __device__ __forceinline__ void block_loss(float a, float b, float c, float* acc
     __syncthreads();
 }
 
-// 1 / x for 1 <= x, and 1 / sqrt(x) with the root itself for x in [1e-16, 1e30):
-// the hardware's approximations with one Newton-Raphson step, which leaves about
-// one unit in the last place, in a third of the instructions of the correctly
-// rounded forms.
+// 1 / x for 1 <= x, and 1 / sqrt(x) for x in [1e-16, 1e30): the hardware's
+// approximations with one Newton-Raphson step.  Over all mantissas the first is
+// 1.0f / x to the bit, the second at most 1.00 units in the last place off
+// (1.0f / sqrtf(x): 1.49).  The root itself is sqrtf: x times the second was up to
+// 0.75 units off and not the nearest in 12 % of the cases.
 __device__ __forceinline__ float reciprocal(float x)
 {
     float r;
@@ -380,13 +381,11 @@ __device__ __forceinline__ float reciprocal(float x)
     return x < 1e30f ? fmaf(r, fmaf(-x, r, 1.0f), r) : r;
 }
 
-__device__ __forceinline__ float inverse_root(float x, float& root)
+__device__ __forceinline__ float inverse_root(float x)
 {
     float r;
     asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    const float h = x * r;              // about the root
-    const float e = fmaf(-h, r, 1.0f);  // 1 - x r^2
-    root = fmaf(0.5f * h, e, h);
+    const float e = fmaf(-(x * r), r, 1.0f);  // 1 - x r^2
     return fmaf(0.5f * r, e, r);
 }
 
@@ -572,12 +571,11 @@ __global__ void __launch_bounds__(T::kThreads, SPARSE ? 2 : 1) sdf_reg_kernel(Sd
                     const float gg = fmaf(g2, g2, fmaf(g1, g1, g0 * g0));
                     const float wn = (SPARSE && !kInner && e[(u + 5) % 6] < 0) ? 0.0f : w;
                     // rho = sqrt(|g|^2 + 1e-24); from 1e-16 on it equals |g| in FP32
-                    float rho, ratio = 1.0f;
-                    float irho = inverse_root(gg, rho), gn = rho;
+                    const float gn = sqrtf(gg);
+                    float rho = gn, ratio = 1.0f, irho = inverse_root(gg);
                     if (!(gg >= 1e-16f && gg < 1e30f)) {
                         rho = sqrtf(gg + 1e-24f);
                         irho = 1.0f / rho;
-                        gn = sqrtf(gg);
                         ratio = gn > 0.0f ? rho / gn : 0.0f;
                     }
                     ir[q] = irho;
