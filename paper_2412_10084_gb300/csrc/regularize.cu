@@ -808,22 +808,27 @@ dim3 dense_domain(const int R[3], int resident, int extra, Domain& D)
     return dim3(tx, ty, (R[2] + D.zc - 1) / D.zc);
 }
 
-// Sparse: a CTA walks kMaxSeg bricks along z, so that neighbouring stored bricks
-// share their halo planes and pipeline (512^3 object, 11 468 stored bricks: all
-// three kernels 1.92 ms with 8, 1.99 ms with 4); with too few bricks to fill the
-// GPU several times over (16 per SM) it takes one.
+// Sparse: a CTA walks up to kMaxSeg bricks along z, so that neighbouring stored
+// bricks share their halo planes and pipeline and fewer CTAs find nothing stored.
+// The number doubles as long as 12 CTAs per SM remain, four times the resident
+// ones: it goes by the table, stored or not, because an empty CTA still costs its
+// launch and its look at the table.  Measured, all three kernels, with 1 / 2 / 4 / 8
+// bricks: 512^3 with 11 468 stored bricks 2.05 / 1.81 / 1.64 / 1.61 ms, 1024^3 with
+// 2400 2.93 / 1.73 / 1.15 / 0.85 ms, 384^3 with 2400 0.55 / 0.47 / 0.46 / 0.46 ms,
+// 256^3 with 2432 442 / 416 / 424 / 454 us, 128^3 with 300 86 / 110 / 138 / 238 us.
 dim3 brick_domain(const int R[3], const int* table, int n_bricks, Domain& D)
 {
-    int64_t entries = 1;
     for (int a = 0; a < 3; ++a) {
         D.R[a] = R[a];
         D.B[a] = R[a] / SB;
-        entries *= D.B[a];
     }
     D.zc = 0;
     D.table = table;
     D.n_bricks = n_bricks;
-    D.seg = n_bricks >= 16 * sms() ? kMaxSeg : 1;
+    const int64_t columns = int64_t(D.B[0]) * D.B[1], enough = 12 * sms();
+    auto ctas = [&](int seg) { return columns * ((D.B[2] + seg - 1) / seg); };
+    D.seg = 1;
+    while (D.seg < kMaxSeg && D.seg < D.B[2] && ctas(2 * D.seg) >= enough) D.seg *= 2;
     return dim3(D.B[0], D.B[1], (D.B[2] + D.seg - 1) / D.seg);
 }
 
