@@ -101,33 +101,45 @@ __device__ __forceinline__ void probe_corner_index(const ProbeView& p, const Cel
 }
 
 // Blended probe coefficients b^_j = sum_i w_i b_ij (Eq. 7 before the SH
-// contraction), two channels per element, the probes in corner order.
-template <class C>
+// contraction), two channels per element, the probes in corner order.  kByRow: the
+// weights and indices of two probes at a time, for the adjoint (28 bytes of spills,
+// 44 with all eight at once); the forward and the shading have the registers for
+// eight (shading of 128^3 nodes 185 us, 190 by rows; the forward the same).
+template <class C, bool kByRow>
 __device__ __forceinline__ void blend_probes(const ProbeView& p, const Cell& pc, float2* B2)
 {
 #pragma unroll
     for (int i = 0; i < C::L2 * C::NA / 2; ++i) B2[i] = make_float2(0.0f, 0.0f);
-    const float x1 = pc.f[0], x0 = 1.0f - x1;
+    auto add = [&](float w, int probe) {
+        const float2 w2 = make_float2(w, w);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const float y = (r & 1) ? pc.f[1] : 1.0f - pc.f[1];
-        const float z = (r & 2) ? pc.f[2] : 1.0f - pc.f[2];
-        const int row = pc.base + ((r & 1) ? p.P[0] : 0) + ((r & 2) ? p.P[0] * p.P[1] : 0);
+        for (int j = 0; j < C::L2; ++j) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const float w = (q ? x1 : x0) * y * z;  // as corner_weights
-            const float2 w2 = make_float2(w, w);
-#pragma unroll
-            for (int j = 0; j < C::L2; ++j) {
-#pragma unroll
-                for (int cg = 0; cg < C::NA4; ++cg) {
-                    const float4 bb = probe_coeffs<C>(p, row + q, j, cg);
-                    float2* b2 = B2 + (j * C::NA + 4 * cg) / 2;
-                    b2[0] = fma2(w2, make_float2(bb.x, bb.y), b2[0]);
-                    b2[1] = fma2(w2, make_float2(bb.z, bb.w), b2[1]);
-                }
+            for (int cg = 0; cg < C::NA4; ++cg) {
+                const float4 bb = probe_coeffs<C>(p, probe, j, cg);
+                float2* b2 = B2 + (j * C::NA + 4 * cg) / 2;
+                b2[0] = fma2(w2, make_float2(bb.x, bb.y), b2[0]);
+                b2[1] = fma2(w2, make_float2(bb.z, bb.w), b2[1]);
             }
         }
+    };
+    if constexpr (kByRow) {
+        const float x1 = pc.f[0], x0 = 1.0f - x1;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float y = (r & 1) ? pc.f[1] : 1.0f - pc.f[1];
+            const float z = (r & 2) ? pc.f[2] : 1.0f - pc.f[2];
+            const int row = pc.base + ((r & 1) ? p.P[0] : 0) + ((r & 2) ? p.P[0] * p.P[1] : 0);
+            add(x0 * y * z, row);  // as corner_weights
+            add(x1 * y * z, row + 1);
+        }
+    } else {
+        float w[8];
+        corner_weights(pc.f, w);
+        int idx[8];
+        probe_corner_index(p, pc, idx);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) add(w[q], idx[q]);
     }
 }
 
@@ -251,7 +263,7 @@ __device__ __forceinline__ void eval_appearance_at(const RenderArgs& A, const fl
         // blended coefficients first (one weight per probe serves all of its
         // coefficients), then F_a = sum_j Y_j b^_j
         float2 B2[C::L2 * C::NA / 2];
-        blend_probes<C>(A.probes, S.pcell, B2);
+        blend_probes<C, false>(A.probes, S.pcell, B2);
 #pragma unroll
         for (int j = 0; j < C::L2; ++j) {
             const float2 y = make_float2(S.Y[j], S.Y[j]);
@@ -343,7 +355,7 @@ __device__ __forceinline__ void eval_appearance_blend(const RenderArgs& A, const
     point_at(o, d, t, xw);
     S.pcell = locate(xw, A.grid.bmin, A.probes.sc, A.probes.P);
     float2 B2[C::L2 * C::NA / 2];
-    blend_probes<C>(A.probes, S.pcell, B2);
+    blend_probes<C, true>(A.probes, S.pcell, B2);
 #pragma unroll
     for (int i = 0; i < C::L2 * C::NA / 2; ++i) {
         Bc[2 * i] = B2[i].x;
