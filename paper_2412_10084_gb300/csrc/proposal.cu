@@ -344,8 +344,8 @@ __device__ __forceinline__ int occ_words(const PropArgs& P)
     return (P.occ_res[0] * P.occ_res[1] * P.occ_res[2] + 31) >> 5;
 }
 
-// Parameters (and, for the adjoint, their accumulators) in static shared
-// memory, the occupancy bitmask in dynamic shared memory.
+// Parameters in static shared memory, the occupancy bitmask in dynamic shared
+// memory.
 template <int B>
 __global__ void proposal_fwd_kernel(PropArgs P)
 {
@@ -767,8 +767,9 @@ PropArgs prop_args(const ProposalLaunch& L)
     return P;
 }
 
-// Static parameter storage plus a bitmask of up to 32 KB can pass the 48 KB
-// default: opt in to the dynamic size the launch needs.
+// A bitmask of up to 32 KB beside the parameters (static) or the adjoint's staging
+// buffer (dynamic) can pass the 48 KB default: opt in to the dynamic size the launch
+// needs.
 template <class K>
 cudaError_t allow_smem(K kernel, size_t dynamic)
 {
