@@ -238,8 +238,8 @@ struct Smooth {
 // Bound: HBM, by the 4-byte SDF slots of the 16-byte records (whole sectors are
 // moved: 0.57 GB for a 256^3 grid).  Measured on 256^3 node records: s 93 us,
 // G^T 95 us (a 32 x 8 x 8 tile with its halo gathered at once: 109 and 155 us);
-// on 47 M stored nodes of a 512^3 grid 297 and 327 us (20^3 tiles gathered per
-// brick with an index division per element: 568 and 763 us).
+// on 47.6 M stored nodes of a 512^3 grid 285 and 302 us (20^3 tiles gathered per
+// brick with an index division per element: 573 and 774 us).
 //
 // Outside the grid the forward reads the replicated edge node and the
 // transpose 0; in an absent brick the forward reads `empty` and the transpose
@@ -433,8 +433,8 @@ struct SdfReg {
 // HBM would take 0.15 ms at 256^3.  s and the own values arrive by asynchronous
 // copies three planes ahead, which cost no registers.  Steps and warps whose
 // columns and planes all lie inside take straight-line code.  Measured: 256^3
-// 0.262 ms (0.421 with three barriers a plane and every neighbour read from
-// shared memory), 47 M stored nodes of a 512^3 grid 1.12 ms (1.28 ms).  Dense
+// 0.268 ms (0.421 with three barriers a plane and every neighbour read from
+// shared memory), 47.6 M stored nodes of a 512^3 grid 1.14 ms (1.29 ms).  Dense
 // tile: 32 x 16 outputs in 864 threads, 1 CTA per SM; 32 x 12 and 32 x 8 with 2
 // CTAs recompute more halo (0.29 and 0.38 ms).
 //

@@ -19,13 +19,13 @@
 // the chunks), one without an opaque sample skips P1-P2 (its weights are all
 // zero).  The log-transmittance carry between chunks uses compensated summation.
 //
-// Bound: the L1 data pipe (76 % of its active cycles: 72 16-byte probe loads a
-// sample, and the CUDA-core layers' parameters from shared memory) and gather
-// latency.  Measured on a 1080p view, 256 samples: 9.6 ms against 9.9 ms with
-// every chunk's opacities evaluated, alpha from an expm1 of its own and two
-// shuffles a value for the one-sample shift.  Layer 1's bias is an FP32 addition
-// on the CUDA cores: as two FP16 columns of the MMA it took 0.15 ms less, but
-// had 22 bits and FP16's range.
+// Bound: the L1 data pipe (71 % of its active cycles, 55 % of the elapsed ones, on
+// 2^14 rays x 256: 72 16-byte probe loads a sample, and the CUDA-core layers'
+// parameters from shared memory) and gather latency.  Measured on a 1080p view, 256
+// samples: 10.2 ms against 10.5 ms with every chunk's opacities evaluated, alpha from
+// an expm1 of its own and two shuffles a value for the one-sample shift.  Layer 1's
+// bias is an FP32 addition on the CUDA cores: as two FP16 columns of the MMA it took
+// 0.18 ms less, but had 22 bits and FP16's range.
 #include "internal.h"
 #include "mlp_tc.cuh"
 
