@@ -371,9 +371,10 @@ __device__ __forceinline__ void block_loss(float a, float b, float c, float* acc
 
 // 1 / x for 1 <= x, and 1 / sqrt(x) for x in [1e-16, 1e30): the hardware's
 // approximations with one Newton-Raphson step.  Over all mantissas the first is
-// 1.0f / x to the bit, the second at most 1.00 units in the last place off
-// (1.0f / sqrtf(x): 1.49).  The root itself is sqrtf: x times the second was up to
-// 0.75 units off and not the nearest in 12 % of the cases.
+// 1.0f / x to the bit below 1e30 (from there on, |s| past 2e29, it is the
+// approximation alone: squares of such values have no FP32), the second at most 1.00
+// units in the last place off (1.0f / sqrtf(x): 1.49).  The root itself is sqrtf: x
+// times the second was up to 0.75 units off and not the nearest in 12 % of the cases.
 __device__ __forceinline__ float reciprocal(float x)
 {
     float r;
